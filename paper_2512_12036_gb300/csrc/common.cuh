@@ -343,6 +343,139 @@ __device__ __forceinline__ int select_bit(unsigned w, int k) {
     return bit;
 }
 
+// warp_expand with the loads of the next kAhead windows of 32 products in
+// flight: load(t) of window w + kAhead is issued before apply(item, a) of
+// window w, a being the A entry's value (kVal) or 0. One copy of each in the
+// loop: an unrolled form with a hash insert in apply overran the instruction
+// cache. The chunk's non-empty segments are moved to the low lanes, so their
+// starts inside a window are distinct and a lane's segment is a popcount of
+// the starts at or before it (one redux.or instead of a five-step shuffle
+// search).
+template <int kAhead, bool kVal, class Load, class Apply>
+__device__ __forceinline__ void warp_expand_ahead(const CsrDev& A, const CsrDev& B, int j0, int j1,
+                                                  Ctl* ctl, Load&& load, Apply&& apply) {
+    using Item = decltype(load(0));
+    const int lane = lane_id();
+    const unsigned le = lanemask_lt() | (1u << lane);
+    for (int base = j0; base < j1; base += 32) {
+        const int j = base + lane;
+        int bs = 0, len = 0;
+        float a = 0.f;
+        if (j < j1) {
+            a_entry(A, B, j, bs, len, ctl);
+            if (kVal) a = A.val[j];
+        }
+        const unsigned ne = __ballot_sync(kFull, len > 0);
+        if (ne & (ne + 1u)) {                       // empty segments in between
+            const int src = select_bit(ne, lane) & 31;
+            bs = __shfl_sync(kFull, bs, src);
+            len = __shfl_sync(kFull, len, src);
+            a = __shfl_sync(kFull, a, src);
+            if (lane >= __popc(ne)) len = 0;
+        }
+        // a chunk too long for 32-bit offsets is walked one segment at a time
+        const bool huge = __any_sync(kFull, len >= kLongRow);
+        int one = 0;
+        do {
+            int mybs = bs, mylen = len;
+            float mya = a;
+            if (huge) {                              // warp-uniform
+                mybs = __shfl_sync(kFull, bs, one);
+                mylen = __shfl_sync(kFull, len, one);
+                mya = __shfl_sync(kFull, a, one);
+                if (lane > 0) mylen = 0;
+            }
+            const unsigned incl = (unsigned)warp_incl_scan(mylen);
+            const unsigned total = __shfl_sync(kFull, incl, 31);
+            const unsigned excl = mylen > 0 ? incl - mylen : 0xffffffffu;   // past every window
+            const int shift = mybs - (int)excl;
+            Item it[kAhead + 1];
+            float av[kAhead + 1];
+            for (unsigned w0 = 0; w0 < total + 32 * kAhead; w0 += 32) {
+#pragma unroll
+                for (int q = 0; q < kAhead; ++q) {
+                    it[q] = it[q + 1];
+                    av[q] = av[q + 1];
+                }
+                if (w0 < total) {                    // warp-uniform
+                    const int first = __popc(__ballot_sync(kFull, excl <= w0)) - 1;
+                    const unsigned rel = excl - w0;
+                    const unsigned starts = __reduce_or_sync(kFull, rel < 32u ? 1u << rel : 0u);
+                    const int s = first + __popc(starts & le & ~1u);
+                    const int t = __shfl_sync(kFull, shift, s) + (int)w0 + lane;
+                    if (kVal) av[kAhead] = __shfl_sync(kFull, mya, s);
+                    if (w0 + lane < total) it[kAhead] = load(t);
+                }
+                if (w0 >= 32 * kAhead && w0 - 32 * kAhead + lane < total) apply(it[0], kVal ? av[0] : 0.f);
+            }
+        } while (huge && ++one < __popc(ne));
+    }
+}
+
+// Ascending sort of 32 * kN keys held by a warp, kN per lane; the sorted
+// order is lane-major (lane l ends with positions l * kN .. l * kN + kN - 1).
+// A bitonic network in registers whose merges begin with the mirrored step,
+// so that every compare-exchange is ascending: strides below kN stay inside
+// a lane, the others are one shuffle per key. The steps across lanes are
+// loops, not unrolled: the whole network of 512 keys is some 2,000
+// instructions and would be fetched anew for every row.
+template <int kN, typename K>
+__device__ __forceinline__ void lane_merge(K (&v)[kN], int half) {
+#pragma unroll
+    for (int j = kN >> 1; j > 0; j >>= 1) {
+        if (j > half) continue;
+#pragma unroll
+        for (int i = 0; i < kN; ++i)
+            if ((i & j) == 0) {
+                const K x = v[i], y = v[i ^ j];
+                v[i] = x < y ? x : y;
+                v[i ^ j] = x < y ? y : x;
+            }
+    }
+}
+
+template <int kN, typename K>
+__device__ __forceinline__ void warp_sort(K (&v)[kN]) {
+    const int lane = lane_id();
+#pragma unroll
+    for (int k = 2; k <= kN; k <<= 1) {
+#pragma unroll
+        for (int i = 0; i < kN; ++i) {
+            const int j = i ^ (k - 1);
+            if (j > i) {
+                const K x = v[i], y = v[j];
+                v[i] = x < y ? x : y;
+                v[j] = x < y ? y : x;
+            }
+        }
+        lane_merge<kN>(v, k >> 2);
+    }
+#pragma unroll 1
+    for (int w = 2; w <= 32; w <<= 1) {              // lanes per merged run
+        {
+            const bool up = (lane & (w >> 1)) != 0;
+#pragma unroll
+            for (int i = 0; i < (kN + 1) / 2; ++i) {
+                const K x = v[i], y = v[kN - 1 - i];
+                const K ox = __shfl_xor_sync(kFull, y, w - 1);
+                const K oy = kN > 1 ? __shfl_xor_sync(kFull, x, w - 1) : ox;
+                v[i] = ((x < ox) != up) ? x : ox;
+                if (kN > 1) v[kN - 1 - i] = ((y < oy) != up) ? y : oy;
+            }
+        }
+#pragma unroll 1
+        for (int m = w >> 2; m > 0; m >>= 1) {
+            const bool up = (lane & m) != 0;
+#pragma unroll
+            for (int i = 0; i < kN; ++i) {
+                const K o = __shfl_xor_sync(kFull, v[i], m);
+                v[i] = ((v[i] < o) != up) ? v[i] : o;
+            }
+        }
+        lane_merge<kN>(v, kN >> 1);
+    }
+}
+
 // Block-wide ordered emit of an occupancy bitmap: the set bits of words
 // [w0, w1) of bm (bit b of word w = column c0 + 32*w + b; bits outside the
 // range to emit must be clear) become entries (column, take(32*w + b)) at

@@ -182,7 +182,15 @@ __device__ __forceinline__ int bin_of(const GroupArgs& g, int r, bool settle) {
     const bool f64 = na > o.fp32_max_terms && ip > o.fp32_max_terms;
     if (ip <= o.esc_max && na <= o.esc_max) return NB_ESC;
     if (g.bcols <= kNarrowCols && ip <= narrow_max_ip(o)) return f64 ? NB_NARROW64 : NB_NARROW32;
-    if (nnz <= o.warp_max_nnz && ip <= 16ll * o.warp_max_nnz) return f64 ? NB_WARP64 : NB_WARP32;
+    if (ip <= 16ll * o.warp_max_nnz) {
+        if (nnz <= o.warp_max_nnz / 2) return f64 ? NB_WARP64S : NB_WARP32S;
+        if (nnz <= o.warp_max_nnz) return f64 ? NB_WARP64 : NB_WARP32;
+        // fp32 rows of up to twice that stay with one warp: a block's barriers
+        // cost a row of this size more than the longer sort of one warp
+        // (131,072 rows of 1,075 products, 600-900 entries: 4,562 us by
+        // 512-thread blocks, 3,827 us by warps)
+        if (!f64 && nnz <= 2 * o.warp_max_nnz && nnz <= o.block_max_nnz) return NB_WARP32L;
+    }
     if (nnz <= block_small_nnz(o)) return f64 ? NB_BLOCK64S : NB_BLOCK32S;
     if (nnz <= block_mid_nnz(o)) return f64 ? NB_BLOCK64M : NB_BLOCK32M;
     if (nnz <= o.block_max_nnz) return f64 ? NB_BLOCK64 : NB_BLOCK32;

@@ -37,7 +37,8 @@ struct spgemm_plan {
     spgemm_opts opts;
     // resident blocks per SM for each persistent kernel (filled at creation)
     int occ_sym_warp, occ_sym_block, occ_sym_dense;
-    int occ_num_warp32, occ_num_warp64, occ_num_block32, occ_num_block64;
+    int occ_num_warp[2][3][2];                // warp tier: fp32/fp64, row size class, wide columns
+    int occ_num_block32, occ_num_block64;
     int occ_num_block32s, occ_num_block64s;   // quarter- and half-size table launches of the block tier
     int occ_num_block32m, occ_num_block64m;
     int occ_num_dense32, occ_num_dense64, occ_num_dense_hot;
@@ -58,7 +59,16 @@ constexpr int kScanItems = 4096;    // rows per block in the row-pointer scan
 constexpr int kWarpTableSym = 2048; // keys per warp, allocation warp tier
 constexpr int kWarpsPerBlockSW = 8;
 constexpr int kWarpTableNum = 1024; // entries per warp, accumulation warp tier
-constexpr int kWarpsPerBlockNW = 8;
+// accumulation warp tier: rows of up to 32 * kN entries, kN = 8, 16 or 32
+// (opts.warp_max_nnz / 2, x 1, x 2 at its default), tables of 64 * kN slots.
+// The largest class takes 7 warps a block: two blocks fill an SM's shared
+// memory with 14 tables of 16 KB (8 warps would leave room for one block).
+constexpr int kWarpClasses[3] = {8, 16, 32};
+__host__ __device__ constexpr int num_warp_warps(int kN) { return kN == 32 ? 7 : 8; }
+__host__ __device__ constexpr int log2_of(int x) { return x <= 1 ? 0 : 1 + log2_of(x / 2); }
+constexpr int kWarpAhead = 2;       // windows of 32 products loaded ahead in the warp tiers
+// widest B whose columns share a 32-bit word with a slot of the largest table
+constexpr int kWarpPackCols = 1 << (32 - 11);
 constexpr int kSymBlockThreads = 512;
 constexpr int kSymDenseThreads = 1024;
 constexpr int kNumBlockThreads = 512;
@@ -78,13 +88,15 @@ constexpr int kMaxPanels = 1024;    // above this the heavy path filters whole B
 //   first), 39/40: block hash fp32/fp64 for rows of at most a quarter of
 //   block_max_nnz entries (a quarter-size table, several blocks per SM),
 //   41/42: the same for rows of at most half (a half-size table),
+//   43/44: warp hash fp32/fp64 for rows of at most half of warp_max_nnz
+//   entries, 45: fp32 for rows of up to twice as many,
 //   63: nothing to do.
 enum : int {
     SB_ESC = 0, SB_WARP = 1, SB_BLOCK0 = 2, SB_BLOCK_N = 4, SB_DENSE0 = 6, SB_DENSE_N = 32,
     NB_ESC = 0, NB_WARP32 = 1, NB_WARP64 = 2, NB_BLOCK32 = 3, NB_BLOCK64 = 4,
     NB_DENSE32_0 = 5, NB_DENSE_N = 16, NB_DENSE64_0 = 21,
     SB_NARROW = 38, NB_NARROW32 = 37, NB_NARROW64 = 38, NB_BLOCK32S = 39, NB_BLOCK64S = 40,
-    NB_BLOCK32M = 41, NB_BLOCK64M = 42
+    NB_BLOCK32M = 41, NB_BLOCK64M = 42, NB_WARP32S = 43, NB_WARP64S = 44, NB_WARP32L = 45
 };
 
 // rows of the accumulation block tier that take the quarter- and half-size

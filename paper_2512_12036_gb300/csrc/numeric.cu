@@ -19,26 +19,24 @@
 
 namespace spg {
 
-template <typename Acc>
-__device__ __forceinline__ void hash_add(int* keys, Acc* vals, int bits, int key, Acc v, Ctl* ctl) {
+// Slot of `key` in an open-addressing table (inserted if new), -1 when the
+// table is full of other keys (never, tables being larger than their rows).
+__device__ __forceinline__ int hash_slot_of(int* keys, int bits, int key, Ctl* ctl) {
     const unsigned mask = (1u << bits) - 1u;
     unsigned h = hash_slot(key, bits);
     for (unsigned probe = 0; probe <= mask; ++probe) {
-        const int cur = *(volatile int*)&keys[h];
-        if (cur == key) {
-            atomicAdd(&vals[h], v);
-            return;
-        }
-        if (cur == kEmpty) {
-            const int old = atomicCAS(&keys[h], kEmpty, key);
-            if (old == kEmpty || old == key) {
-                atomicAdd(&vals[h], v);
-                return;
-            }
-        }
+        const int old = atomicCAS(&keys[h], kEmpty, key);
+        if (old == kEmpty || old == key) return (int)h;
         h = (h + 1u) & mask;
     }
     set_status(ctl, ST_INTERNAL);
+    return -1;
+}
+
+template <typename Acc>
+__device__ __forceinline__ void hash_add(int* keys, Acc* vals, int bits, int key, Acc v, Ctl* ctl) {
+    const int h = hash_slot_of(keys, bits, key, ctl);
+    if (h >= 0) atomicAdd(&vals[h], v);
 }
 
 struct KeyVal {
@@ -229,24 +227,85 @@ __device__ bool block_bucket_sort(int* keys, Acc* vals, int n, int off, int* cnt
     return true;
 }
 
-template <typename Acc>
-__global__ void __launch_bounds__(kWarpsPerBlockNW * 32) k_num_warp(CsrDev A, CsrDev B,
-                                                                    const int* map, Ctl* ctl,
-                                                                    const int* rptC, int row_begin,
-                                                                    int* colC, float* valC,
-                                                                    int bin, int load_pct) {
+// Sort n <= 32 * kN packed keys keys[0, n) of a warp's table in registers and
+// leave them sorted at keys[t + t / 32] (the gap spreads the lane-major order
+// of warp_sort over the banks).
+template <int kN>
+__device__ __forceinline__ void warp_sort_packed(int* keys, int n) {
+    const int lane = lane_id();
+    unsigned v[kN];
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+        const int t = lane + 32 * i;
+        v[i] = t < n ? (unsigned)keys[t] : 0xffffffffu;
+    }
+    warp_sort<kN>(v);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+        const int t = lane * kN + i;
+        if (t < n) keys[t + (t >> 5)] = (int)v[i];
+    }
+    __syncwarp();
+}
+
+// The same for columns too wide to share 32 bits with a slot: the sorted
+// (column, slot) pairs go straight to out(position, column, slot).
+template <int kN, class Out>
+__device__ __forceinline__ void warp_sort_wide(const int* keys, int T, int n, Out&& out) {
+    const int lane = lane_id();
+    unsigned long long v[kN];
+    // slots are taken in table order: entry q of the table's occupied slots
+    // (compacted list keys[0, n) of slots kept at keys[T ..] by the caller)
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+        const int t = lane + 32 * i;
+        v[i] = ~0ull;
+        if (t < n) {
+            const int slot = keys[T + t];
+            v[i] = ((unsigned long long)(unsigned)keys[slot] << 32) | (unsigned)slot;
+        }
+    }
+    warp_sort<kN>(v);
+#pragma unroll
+    for (int i = 0; i < kN; ++i) {
+        const int t = lane * kN + i;
+        if (t < n) out(t, (int)(v[i] >> 32), (int)(v[i] & 0xffffffffu));
+    }
+}
+
+// Warp hash tier. One warp per row: products are added into an open-addressing
+// table in shared memory, the occupied slots are compacted to (column, slot)
+// pairs and sorted in registers, and the row is written in column order, the
+// values fetched from their slots. What bounds it is instruction issue (420
+// warp instructions per 32 products, 1,530 with a bitonic network on the
+// table in shared memory; 100,003 rows of 256 products: 1,962 -> 692 us). A
+// pair is one 32-bit word when B's columns fit 32 - 11 bits (kWide = false),
+// else two. kN: entries per lane the sort may hold (rows of up to 32 * kN entries,
+// tables of up to 64 * kN slots); rows are launched by that size, so that the
+// smaller tables leave room for more warps.
+template <typename Acc, int kN, bool kWide>
+__global__ void __launch_bounds__(num_warp_warps(kN) * 32) k_num_warp(
+    CsrDev A, CsrDev B, const int* map, Ctl* ctl, const int* rptC, int row_begin, int* colC,
+    float* valC, int bin, int load_pct) {
+    constexpr int kWarps = num_warp_warps(kN);
+    constexpr int kTab = 64 * kN;
+    constexpr int kMaxBits = log2_of(kTab);
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int warp = threadIdx.x >> 5, lane = lane_id();
-    Acc* vals = reinterpret_cast<Acc*>(sm_raw) + warp * kWarpTableNum;
-    int* keys = reinterpret_cast<int*>(sm_raw + sizeof(Acc) * kWarpsPerBlockNW * kWarpTableNum) +
-                warp * kWarpTableNum;
+    Acc* vals = reinterpret_cast<Acc*>(sm_raw) + warp * kTab;
+    int* keys = reinterpret_cast<int*>(sm_raw + sizeof(Acc) * kWarps * kTab) +
+                warp * (kWide ? kTab + kTab / 2 : kTab);
     const int begin = ctl->bin_off[bin], end = ctl->bin_off[bin + 1];
     const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
-    constexpr int kMaxBits = 10;
+    int r_next = begin + gw < end ? map[begin + gw] : 0;
     for (int idx = begin + gw; idx < end; idx += nw) {
-        const int r = map[idx];
+        const int r = r_next;
+        if (idx + nw < end) r_next = map[idx + nw];
         const int row = row_begin + r;
+        int rs, re;
+        row_extent(A, row, rs, re, ctl);
         const int out = rptC[r];
         const int nnz_row = rptC[r + 1] - out;
         const int bits = table_bits(nnz_row, load_pct, 5, kMaxBits);
@@ -256,38 +315,44 @@ __global__ void __launch_bounds__(kWarpsPerBlockNW * 32) k_num_warp(CsrDev A, Cs
             vals[t] = Acc(0);
         }
         __syncwarp();
-        int rs, re;
-        row_extent(A, row, rs, re, ctl);
-        warp_expand(A, B, rs, re, 32, ctl, [&](int t, int ja) {
-            const int key = B.col[t];
-            if (key_in(key, B, ctl))
-                hash_add<Acc>(keys, vals, bits, key, (Acc)A.val[ja] * (Acc)B.val[t], ctl);
-        });
+        warp_expand_ahead<kWarpAhead, true>(
+            A, B, rs, re, ctl, [&](int t) { return KeyVal{B.col[t], B.val[t]}; },
+            [&](KeyVal kv, float a) {
+                if (key_in(kv.key, B, ctl)) hash_add<Acc>(keys, vals, bits, kv.key, (Acc)a * (Acc)kv.v, ctl);
+            });
         __syncwarp();
         int n = 0;
         for (int c = 0; c < T; c += 32) {
             const int k = keys[c + lane];
-            const Acc v = vals[c + lane];
             const bool occ = k != kEmpty;
             const unsigned bal = __ballot_sync(kFull, occ);
-            const int pos = n + __popc(bal & lanemask_lt());
-            __syncwarp();
             if (occ) {
-                keys[pos] = k;
-                vals[pos] = v;
+                const int pos = n + __popc(bal & lanemask_lt());
+                if (!kWide) keys[pos] = (int)(((unsigned)k << bits) | (unsigned)(c + lane));
+                else if (pos < kTab / 2) keys[T + pos] = c + lane;
             }
             n += __popc(bal);
             __syncwarp();
         }
         if (lane == 0 && n != nnz_row) set_status(ctl, ST_INTERNAL);
         const int nn = n < nnz_row ? n : nnz_row;
-        const int n2 = (int)pow2_ceil((unsigned)(nn > 1 ? nn : 1));
-        for (int t = nn + lane; t < n2; t += 32) keys[t] = 0x7fffffff;
-        __syncwarp();
-        bitonic_sort<Acc, false>(keys, vals, n2, lane, 32);
-        for (int t = lane; t < nn; t += 32) {
-            colC[out + t] = keys[t];
-            valC[out + t] = (float)vals[t];
+        if constexpr (kWide) {
+            auto put = [&](int t, int col, int slot) {
+                colC[out + t] = col;
+                valC[out + t] = (float)vals[slot];
+            };
+            if (kN == 8 && nn <= 64) warp_sort_wide<2>(keys, T, nn, put);
+            else warp_sort_wide<kN>(keys, T, nn, put);
+        } else {
+            // (the larger classes hold no shorter rows)
+            if (kN == 8 && nn <= 64) warp_sort_packed<2>(keys, nn);
+            else if (kN == 8 && nn <= 128) warp_sort_packed<4>(keys, nn);
+            else warp_sort_packed<kN>(keys, nn);
+            for (int t = lane; t < nn; t += 32) {
+                const unsigned pk = (unsigned)keys[t + (t >> 5)];
+                colC[out + t] = (int)(pk >> bits);
+                valC[out + t] = (float)vals[pk & (unsigned)(T - 1)];
+            }
         }
         __syncwarp();
     }
@@ -1640,7 +1705,15 @@ constexpr size_t hot_smem_of(int pw, int ppp) {
 
 // ---------------------------------------------------------------------------
 
-static size_t num_warp_smem(size_t acc) { return (acc + 4) * kWarpsPerBlockNW * kWarpTableNum; }
+static size_t num_warp_smem(size_t acc, int kN, bool wide) {
+    return (acc + (wide ? 6 : 4)) * (size_t)num_warp_warps(kN) * 64 * kN;
+}
+
+template <typename Acc, int kN, class F>
+static void num_warp_kernel(bool wide, F&& f) {
+    if (wide) f((const void*)k_num_warp<Acc, kN, true>, k_num_warp<Acc, kN, true>);
+    else f((const void*)k_num_warp<Acc, kN, false>, k_num_warp<Acc, kN, false>);
+}
 static size_t num_block_smem(const spgemm_plan* p, size_t acc) {
     return (acc + 4) * pow2_ceil(2u * (unsigned)p->opts.block_max_nnz);
 }
@@ -1750,8 +1823,6 @@ void occupancy_numeric(spgemm_plan* p) {
     } ks[] = {
         {(const void*)k_num_dense_rank, kRankThreads, rank_smem(p, kRankPanels, p->opts.panel_cols),
          &p->occ_num_rank},
-        {(const void*)k_num_warp<float>, kWarpsPerBlockNW * 32, num_warp_smem(4), &p->occ_num_warp32},
-        {(const void*)k_num_warp<double>, kWarpsPerBlockNW * 32, num_warp_smem(8), &p->occ_num_warp64},
         {(const void*)k_num_block<float, kBlockThreadsFull>, kBlockThreadsFull, num_block_smem(p, 4),
          &p->occ_num_block32},
         {(const void*)k_num_block<double, kBlockThreadsFull>, kBlockThreadsFull, num_block_smem(p, 8),
@@ -1764,6 +1835,21 @@ void occupancy_numeric(spgemm_plan* p) {
         {(const void*)k_num_dense<1, 1024>, 1024, num_dense_smem(p, 1), &p->occ_num_dense64},
         {(const void*)k_num_dense_hot, kHotThreads, num_dense_hot_smem(p), &p->occ_num_dense_hot},
     };
+    auto warp_occ = [&](const void* f, size_t acc, int cls, bool wide) {
+        allow_max_dynamic_smem(f, p);
+        const int kN = kWarpClasses[cls];
+        int* occ = &p->occ_num_warp[acc == 8][cls][wide];
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, f, num_warp_warps(kN) * 32,
+                                                      num_warp_smem(acc, kN, wide));
+        if (*occ < 1) *occ = 1;
+    };
+    for (int wide = 0; wide < 2; ++wide) {
+        num_warp_kernel<float, 8>(wide, [&](const void* f, auto) { warp_occ(f, 4, 0, wide); });
+        num_warp_kernel<float, 16>(wide, [&](const void* f, auto) { warp_occ(f, 4, 1, wide); });
+        num_warp_kernel<float, 32>(wide, [&](const void* f, auto) { warp_occ(f, 4, 2, wide); });
+        num_warp_kernel<double, 8>(wide, [&](const void* f, auto) { warp_occ(f, 8, 0, wide); });
+        num_warp_kernel<double, 16>(wide, [&](const void* f, auto) { warp_occ(f, 8, 1, wide); });
+    }
     allow_max_dynamic_smem((const void*)k_num_narrow<float>, p);
     allow_max_dynamic_smem((const void*)k_num_narrow<double>, p);
     for (auto& k : ks) {
@@ -1853,12 +1939,21 @@ void launch_numeric(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, cons
                    k_num_narrow<double><<<grid, nwp * 32, (size_t)nwp * (pad * 8 + 128), s>>>(
                        A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_NARROW64, pad));
     }
-    SPG_LAUNCH(p, K_NUM_WARP32, s,
-               k_num_warp<float><<<sms * p->occ_num_warp32, kWarpsPerBlockNW * 32, num_warp_smem(4), s>>>(
-                   A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_WARP32, hash_load(p)));
-    SPG_LAUNCH(p, K_NUM_WARP64, s,
-               k_num_warp<double><<<sms * p->occ_num_warp64, kWarpsPerBlockNW * 32, num_warp_smem(8), s>>>(
-                   A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_WARP64, hash_load(p)));
+    const bool wide = B.cols > kWarpPackCols;
+    auto warp_tier = [&](int kid, size_t acc, int cls, int bin) {
+        return [=](const void*, auto kernel) {
+            const int kN = kWarpClasses[cls];
+            SPG_LAUNCH(p, kid, s,
+                       kernel<<<sms * p->occ_num_warp[acc == 8][cls][wide], num_warp_warps(kN) * 32,
+                                num_warp_smem(acc, kN, wide), s>>>(
+                           A, B, w.map, w.ctl, rptC, row_begin, colC, valC, bin, hash_load(p)));
+        };
+    };
+    num_warp_kernel<float, 32>(wide, warp_tier(K_NUM_WARP32, 4, 2, NB_WARP32L));
+    num_warp_kernel<float, 16>(wide, warp_tier(K_NUM_WARP32, 4, 1, NB_WARP32));
+    num_warp_kernel<float, 8>(wide, warp_tier(K_NUM_WARP32, 4, 0, NB_WARP32S));
+    num_warp_kernel<double, 16>(wide, warp_tier(K_NUM_WARP64, 8, 1, NB_WARP64));
+    num_warp_kernel<double, 8>(wide, warp_tier(K_NUM_WARP64, 8, 0, NB_WARP64S));
     // block hash tier: rows of more than half of block_max_nnz entries with
     // the full table (one block per SM), the others with a half- or
     // quarter-size table and as many blocks per SM as it leaves room for
