@@ -51,6 +51,11 @@ __device__ __forceinline__ unsigned lanemask_lt() {
     return m;
 }
 
+template <int kV>
+struct IntC {
+    static constexpr int value = kV;
+};
+
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {
 #pragma unroll
@@ -344,19 +349,22 @@ __device__ __forceinline__ int select_bit(unsigned w, int k) {
 }
 
 // warp_expand with the loads of the next kAhead windows of 32 products in
-// flight: load(t) of window w + kAhead is issued before apply(item, a) of
-// window w, a being the A entry's value (kVal) or 0. One copy of each in the
+// flight: load(t) of window w + kAhead is issued before apply(item, a, q) of
+// window w, a being the A entry's value (kVal) or 0 and q the product's
+// position in the row. Returns the row's products. One copy of each in the
 // loop: an unrolled form with a hash insert in apply overran the instruction
 // cache. The chunk's non-empty segments are moved to the low lanes, so their
 // starts inside a window are distinct and a lane's segment is a popcount of
 // the starts at or before it (one redux.or instead of a five-step shuffle
 // search).
 template <int kAhead, bool kVal, class Load, class Apply>
-__device__ __forceinline__ void warp_expand_ahead(const CsrDev& A, const CsrDev& B, int j0, int j1,
-                                                  Ctl* ctl, Load&& load, Apply&& apply) {
+__device__ __forceinline__ unsigned warp_expand_ahead(const CsrDev& A, const CsrDev& B, int j0,
+                                                      int j1, Ctl* ctl, Load&& load,
+                                                      Apply&& apply) {
     using Item = decltype(load(0));
     const int lane = lane_id();
     const unsigned le = lanemask_lt() | (1u << lane);
+    unsigned done = 0;
     for (int base = j0; base < j1; base += 32) {
         const int j = base + lane;
         int bs = 0, len = 0;
@@ -406,10 +414,13 @@ __device__ __forceinline__ void warp_expand_ahead(const CsrDev& A, const CsrDev&
                     if (kVal) av[kAhead] = __shfl_sync(kFull, mya, s);
                     if (w0 + lane < total) it[kAhead] = load(t);
                 }
-                if (w0 >= 32 * kAhead && w0 - 32 * kAhead + lane < total) apply(it[0], kVal ? av[0] : 0.f);
+                const unsigned p = w0 - 32 * kAhead + lane;
+                if (w0 >= 32 * kAhead && p < total) apply(it[0], kVal ? av[0] : 0.f, done + p);
             }
+            done += total;
         } while (huge && ++one < __popc(ne));
     }
+    return done;
 }
 
 // Ascending sort of 32 * kN keys held by a warp, kN per lane; the sorted

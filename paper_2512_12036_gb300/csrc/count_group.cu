@@ -169,6 +169,7 @@ __device__ __forceinline__ int bin_of(const GroupArgs& g, int r, bool settle) {
         }
         if (ip <= o.esc_max && na <= o.esc_max) return SB_ESC;
         if (g.bcols <= kNarrowCols && ip <= narrow_max_ip(o)) return SB_NARROW;
+        if (ip <= sort_max_ip(o.warp_max_ip / 2)) return ip <= sort_max_ip(o.warp_max_ip / 2) / 2 ? SB_SORTA : SB_SORTB;
         if (ip <= o.warp_max_ip) return SB_WARP;
         const int L = log2_ceil_ll(ip);
         if (ip <= o.block_max_ip) {
@@ -182,6 +183,10 @@ __device__ __forceinline__ int bin_of(const GroupArgs& g, int r, bool settle) {
     const bool f64 = na > o.fp32_max_terms && ip > o.fp32_max_terms;
     if (ip <= o.esc_max && na <= o.esc_max) return NB_ESC;
     if (g.bcols <= kNarrowCols && ip <= narrow_max_ip(o)) return f64 ? NB_NARROW64 : NB_NARROW32;
+    if (ip <= sort_max_ip(o.warp_max_nnz) && g.bcols < kSortCols) {
+        if (ip <= sort_max_ip(o.warp_max_nnz) / 2) return f64 ? NB_SORT64A : NB_SORT32A;
+        return f64 ? NB_SORT64B : NB_SORT32B;
+    }
     if (ip <= 16ll * o.warp_max_nnz) {
         if (nnz <= o.warp_max_nnz / 2) return f64 ? NB_WARP64S : NB_WARP32S;
         if (nnz <= o.warp_max_nnz) return f64 ? NB_WARP64 : NB_WARP32;

@@ -37,6 +37,7 @@ struct spgemm_plan {
     spgemm_opts opts;
     // resident blocks per SM for each persistent kernel (filled at creation)
     int occ_sym_warp, occ_sym_block, occ_sym_dense;
+    int occ_sym_sort[2], occ_num_sort[2][2];  // sort tier: size class (fp32/fp64 first)
     int occ_num_warp[2][3][2];                // warp tier: fp32/fp64, row size class, wide columns
     int occ_num_block32, occ_num_block64;
     int occ_num_block32s, occ_num_block64s;   // quarter- and half-size table launches of the block tier
@@ -66,6 +67,11 @@ constexpr int kWarpTableNum = 1024; // entries per warp, accumulation warp tier
 constexpr int kWarpClasses[3] = {8, 16, 32};
 __host__ __device__ constexpr int num_warp_warps(int kN) { return kN == 32 ? 7 : 8; }
 __host__ __device__ constexpr int log2_of(int x) { return x <= 1 ? 0 : 1 + log2_of(x / 2); }
+// sort tier: rows of up to 32 * kN products (kN = 8, 16) sorted in registers
+constexpr int kSortWarps = 8;
+constexpr int kSortCols = 1 << 23;  // accumulation: B's columns stay below (a 32-bit word holds
+                                    // a column and a product's position)
+__host__ __device__ inline int sort_max_ip(int limit) { return limit < 512 ? limit : 512; }
 constexpr int kWarpAhead = 2;       // windows of 32 products loaded ahead in the warp tiers
 // widest B whose columns share a 32-bit word with a slot of the largest table
 constexpr int kWarpPackCols = 1 << (32 - 11);
@@ -81,7 +87,8 @@ constexpr int kMaxPanels = 1024;    // above this the heavy path filters whole B
 
 // Bins (phase-specific meaning). Allocation phase:
 //   0: in-register tier, 1: warp hash, 2..5: block hash (by log2 IP, heavy
-//   first), 6..37: dense bitmap (by log2 IP, heavy first), 63: nothing to do.
+//   first), 6..37: dense bitmap (by log2 IP, heavy first), 38: narrow,
+//   39/40: sort tier, up to 256 and 512 products, 63: nothing to do.
 // Accumulation phase:
 //   0: in-register tier, 1/2: warp hash fp32/fp64, 3/4: block hash fp32/fp64,
 //   5..20: dense panels fp32, 21..36: dense panels fp64 (by log2 IP, heavy
@@ -89,14 +96,17 @@ constexpr int kMaxPanels = 1024;    // above this the heavy path filters whole B
 //   block_max_nnz entries (a quarter-size table, several blocks per SM),
 //   41/42: the same for rows of at most half (a half-size table),
 //   43/44: warp hash fp32/fp64 for rows of at most half of warp_max_nnz
-//   entries, 45: fp32 for rows of up to twice as many,
+//   entries, 45: fp32 for rows of up to twice as many, 46/47 and 48/49: sort
+//   tier fp32 and fp64, rows of up to 256 and 512 products,
 //   63: nothing to do.
 enum : int {
     SB_ESC = 0, SB_WARP = 1, SB_BLOCK0 = 2, SB_BLOCK_N = 4, SB_DENSE0 = 6, SB_DENSE_N = 32,
     NB_ESC = 0, NB_WARP32 = 1, NB_WARP64 = 2, NB_BLOCK32 = 3, NB_BLOCK64 = 4,
     NB_DENSE32_0 = 5, NB_DENSE_N = 16, NB_DENSE64_0 = 21,
     SB_NARROW = 38, NB_NARROW32 = 37, NB_NARROW64 = 38, NB_BLOCK32S = 39, NB_BLOCK64S = 40,
-    NB_BLOCK32M = 41, NB_BLOCK64M = 42, NB_WARP32S = 43, NB_WARP64S = 44, NB_WARP32L = 45
+    NB_BLOCK32M = 41, NB_BLOCK64M = 42, NB_WARP32S = 43, NB_WARP64S = 44, NB_WARP32L = 45,
+    NB_SORT32A = 46, NB_SORT32B = 47, NB_SORT64A = 48, NB_SORT64B = 49,
+    SB_SORTA = 39, SB_SORTB = 40
 };
 
 // rows of the accumulation block tier that take the quarter- and half-size
