@@ -8,6 +8,7 @@
 namespace spg {
 void occupancy_symbolic(spgemm_plan* p);
 void occupancy_numeric(spgemm_plan* p);
+void occupancy_bits(spgemm_plan* p);
 void occupancy_backward(spgemm_plan* p);
 void occupancy_mcl(spgemm_plan* p);
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -112,6 +113,7 @@ void allow_max_dynamic_smem(const void* f, const spgemm_plan* p) {
 void init_occupancy(spgemm_plan* p) {
     occupancy_symbolic(p);
     occupancy_numeric(p);
+    occupancy_bits(p);
     occupancy_backward(p);
     occupancy_mcl(p);
 }

@@ -72,6 +72,11 @@ constexpr int kSortWarps = 8;
 constexpr int kSortCols = 1 << 23;  // accumulation: B's columns stay below (a 32-bit word holds
                                     // a column and a product's position)
 __host__ __device__ inline int sort_max_ip(int limit) { return limit < 512 ? limit : 512; }
+// bitmap tiers: columns of B at most; shared memory of an SM, and what a
+// block of theirs holds beside its dynamic part at most
+constexpr int kBitsCols = 1 << 19;
+constexpr size_t kBitsSmem = 228 * 1024;
+constexpr size_t kBitsStatic = 8 * 1024;
 constexpr int kWarpAhead = 2;       // windows of 32 products loaded ahead in the warp tiers
 // widest B whose columns share a 32-bit word with a slot of the largest table
 constexpr int kWarpPackCols = 1 << (32 - 11);
@@ -90,23 +95,23 @@ constexpr int kMaxPanels = 1024;    // above this the heavy path filters whole B
 //   first), 6..37: dense bitmap (by log2 IP, heavy first), 38: narrow,
 //   39/40: sort tier, up to 256 and 512 products, 63: nothing to do.
 // Accumulation phase:
-//   0: in-register tier, 1/2: warp hash fp32/fp64, 3/4: block hash fp32/fp64,
-//   5..20: dense panels fp32, 21..36: dense panels fp64 (by log2 IP, heavy
-//   first), 39/40: block hash fp32/fp64 for rows of at most a quarter of
-//   block_max_nnz entries (a quarter-size table, several blocks per SM),
-//   41/42: the same for rows of at most half (a half-size table),
-//   43/44: warp hash fp32/fp64 for rows of at most half of warp_max_nnz
-//   entries, 45: fp32 for rows of up to twice as many, 46/47 and 48/49: sort
-//   tier fp32 and fp64, rows of up to 256 and 512 products,
+//   0: in-register tier, 1: fp32 rows of more than block_max_nnz entries that
+//   the bitmap tier takes, 5..20: dense panels fp32, 21..36: dense panels
+//   fp64 (by log2 IP, heavy first), 37/38: narrow fp32/fp64,
+//   39..41: warp hash fp32 by row size (up to half of warp_max_nnz entries,
+//   up to it, up to twice it), 42..44: block hash fp32 (up to a quarter of
+//   block_max_nnz, a half, all), 45..46 and 47..49: the same for fp64 (rows of
+//   39..49 go to the bitmap tier where B is narrow enough for it),
+//   50/51 and 52/53: sort tier fp32 and fp64 (up to 256 and 512 products),
 //   63: nothing to do.
 enum : int {
     SB_ESC = 0, SB_WARP = 1, SB_BLOCK0 = 2, SB_BLOCK_N = 4, SB_DENSE0 = 6, SB_DENSE_N = 32,
-    NB_ESC = 0, NB_WARP32 = 1, NB_WARP64 = 2, NB_BLOCK32 = 3, NB_BLOCK64 = 4,
-    NB_DENSE32_0 = 5, NB_DENSE_N = 16, NB_DENSE64_0 = 21,
-    SB_NARROW = 38, NB_NARROW32 = 37, NB_NARROW64 = 38, NB_BLOCK32S = 39, NB_BLOCK64S = 40,
-    NB_BLOCK32M = 41, NB_BLOCK64M = 42, NB_WARP32S = 43, NB_WARP64S = 44, NB_WARP32L = 45,
-    NB_SORT32A = 46, NB_SORT32B = 47, NB_SORT64A = 48, NB_SORT64B = 49,
-    SB_SORTA = 39, SB_SORTB = 40
+    SB_NARROW = 38, SB_SORTA = 39, SB_SORTB = 40,
+    NB_ESC = 0, NB_BITS32 = 1, NB_DENSE32_0 = 5, NB_DENSE_N = 16, NB_DENSE64_0 = 21,
+    NB_NARROW32 = 37, NB_NARROW64 = 38,
+    NB_WARP32S = 39, NB_WARP32 = 40, NB_WARP32L = 41, NB_BLOCK32S = 42, NB_BLOCK32M = 43, NB_BLOCK32 = 44,
+    NB_WARP64S = 45, NB_WARP64 = 46, NB_BLOCK64S = 47, NB_BLOCK64M = 48, NB_BLOCK64 = 49,
+    NB_SORT32A = 50, NB_SORT32B = 51, NB_SORT64A = 52, NB_SORT64B = 53
 };
 
 // rows of the accumulation block tier that take the quarter- and half-size
@@ -206,6 +211,7 @@ struct GroupArgs {
     int nthr;
     int bcols;                 // columns of B (narrow tiers, backward dense tier)
     const int* rc_slot;        // accumulation: row bitmap cache slots, or nullptr
+    int bits_cap;              // accumulation: entries of an fp32 bitmap-tier row at most (0: no such tier)
     spgemm_opts opts;
 };
 void launch_group(const spgemm_plan* p, const GroupArgs& g, const WsPtrs& w, int* map_out,
@@ -223,6 +229,14 @@ void launch_nnz_total(const spgemm_plan* p, const int* row_nnz, int n, const WsP
 void launch_numeric(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const long long* ip,
                     int row_begin, int row_end, const int* rptC, const WsPtrs& w, int* colC,
                     float* valC, cudaStream_t s, long long capacity = -1);
+// Bitmap tiers (bits.cu).
+bool bits_tier(const spgemm_plan* p, const CsrDev& B);
+int bits_cap(const spgemm_plan* p, const CsrDev& B, size_t acc);
+void launch_sym_bits(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const WsPtrs& w,
+                     int* row_nnz, int bin_lo, int bin_hi, int tier, cudaStream_t s);
+void launch_num_bits(const spgemm_plan* p, bool f64, const CsrDev& A, const CsrDev& B, const WsPtrs& w,
+                     const int* rptC, int row_begin, int* colC, float* valC, int bin_lo, int bin_hi,
+                     int tier, int cap, cudaStream_t s);
 void launch_bpanel(const spgemm_plan* p, const CsrDev& B, const WsPtrs& w, cudaStream_t s);
 void launch_hot(const spgemm_plan* p, const CsrDev& B, const WsPtrs& w, cudaStream_t s);
 void launch_copy_total(const spgemm_plan* p, const WsPtrs& w, int which, long long* dst,

@@ -1998,46 +1998,11 @@ static int dense_splits(const spgemm_plan* p, int panels) {
     return sp;
 }
 
-void launch_numeric(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const long long* ip,
-                    int row_begin, int row_end, const int* rptC, const WsPtrs& w, int* colC,
-                    float* valC, cudaStream_t s, long long capacity) {
-    GroupArgs g{};
-    g.phase = 1;
-    g.row_begin = row_begin;
-    g.n = row_end - row_begin;
-    g.ip = ip;
-    g.rptA = A.rpt;
-    g.rptC = rptC;
-    g.bcols = B.cols;
-    g.rc_slot = w.rc_slot;
-    g.opts = p->opts;
-    launch_group(p, g, w, w.map, nullptr, s);
-    if (g.n == 0) return;
-    if (capacity >= 0)
-        SPG_LAUNCH(p, K_GUARD, s, k_cap_guard<<<1, 64, 0, s>>>(rptC, g.n, capacity, w.ctl));
+// Warp and block hash tiers: rows that outgrow the sort tier, for a B too
+// wide (or too narrow) for the bitmap tier.
+static void launch_num_hash(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const int* rptC,
+                            int row_begin, const WsPtrs& w, int* colC, float* valC, cudaStream_t s) {
     const int sms = p->num_sms;
-    SPG_LAUNCH(p, K_NUM_ESC, s, k_num_esc<<<sms * 8, 256, 0, s>>>(A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_ESC));
-    if (B.cols <= kNarrowCols) {
-        const int pad = (B.cols + 31) & ~31;
-        const int nwp = narrow_warps(p);
-        const int grid = sms * (64 / nwp > 1 ? 64 / nwp : 1);
-        SPG_LAUNCH(p, K_NUM_NARROW, s,
-                   k_num_narrow<float><<<grid, nwp * 32, (size_t)nwp * (pad * 4 + 128), s>>>(
-                       A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_NARROW32, pad));
-        SPG_LAUNCH(p, K_NUM_NARROW, s,
-                   k_num_narrow<double><<<grid, nwp * 32, (size_t)nwp * (pad * 8 + 128), s>>>(
-                       A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_NARROW64, pad));
-    }
-    if (B.cols < kSortCols) {
-        auto sort_tier = [&](int kid, auto kernel, int occ, int bin) {
-            SPG_LAUNCH(p, kid, s, kernel<<<sms * occ, kSortWarps * 32, 0, s>>>(
-                A, B, w.map, w.ctl, rptC, row_begin, colC, valC, bin));
-        };
-        sort_tier(K_NUM_WARP32, k_num_sort<float, 16>, p->occ_num_sort[0][1], NB_SORT32B);
-        sort_tier(K_NUM_WARP32, k_num_sort<float, 8>, p->occ_num_sort[0][0], NB_SORT32A);
-        sort_tier(K_NUM_WARP64, k_num_sort<double, 16>, p->occ_num_sort[1][1], NB_SORT64B);
-        sort_tier(K_NUM_WARP64, k_num_sort<double, 8>, p->occ_num_sort[1][0], NB_SORT64A);
-    }
     const bool wide = B.cols > kWarpPackCols;
     auto warp_tier = [&](int kid, size_t acc, int cls, int bin) {
         return [=](const void*, auto kernel) {
@@ -2085,6 +2050,66 @@ void launch_numeric(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, cons
                k_num_block<double><<<sms * p->occ_num_block64s, kNumBlockThreads, num_block_smem_small(p, 8), s>>>(
                    A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_BLOCK64S, 9, small_bits,
                    hash_load(p)));
+}
+
+void launch_numeric(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const long long* ip,
+                    int row_begin, int row_end, const int* rptC, const WsPtrs& w, int* colC,
+                    float* valC, cudaStream_t s, long long capacity) {
+    GroupArgs g{};
+    g.phase = 1;
+    g.row_begin = row_begin;
+    g.n = row_end - row_begin;
+    g.ip = ip;
+    g.rptA = A.rpt;
+    g.rptC = rptC;
+    g.bcols = B.cols;
+    g.rc_slot = w.rc_slot;
+    // rows with cached bitmaps stay in the dense tiers, which read them
+    g.bits_cap = bits_tier(p, B) && !w.rc_slot ? bits_cap(p, B, sizeof(float)) : 0;
+    g.opts = p->opts;
+    launch_group(p, g, w, w.map, nullptr, s);
+    if (g.n == 0) return;
+    if (capacity >= 0)
+        SPG_LAUNCH(p, K_GUARD, s, k_cap_guard<<<1, 64, 0, s>>>(rptC, g.n, capacity, w.ctl));
+    const int sms = p->num_sms;
+    SPG_LAUNCH(p, K_NUM_ESC, s, k_num_esc<<<sms * 8, 256, 0, s>>>(A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_ESC));
+    if (B.cols <= kNarrowCols) {
+        const int pad = (B.cols + 31) & ~31;
+        const int nwp = narrow_warps(p);
+        const int grid = sms * (64 / nwp > 1 ? 64 / nwp : 1);
+        SPG_LAUNCH(p, K_NUM_NARROW, s,
+                   k_num_narrow<float><<<grid, nwp * 32, (size_t)nwp * (pad * 4 + 128), s>>>(
+                       A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_NARROW32, pad));
+        SPG_LAUNCH(p, K_NUM_NARROW, s,
+                   k_num_narrow<double><<<grid, nwp * 32, (size_t)nwp * (pad * 8 + 128), s>>>(
+                       A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_NARROW64, pad));
+    }
+    if (B.cols < kSortCols) {
+        auto sort_tier = [&](int kid, auto kernel, int occ, int bin) {
+            SPG_LAUNCH(p, kid, s, kernel<<<sms * occ, kSortWarps * 32, 0, s>>>(
+                A, B, w.map, w.ctl, rptC, row_begin, colC, valC, bin));
+        };
+        sort_tier(K_NUM_WARP32, k_num_sort<float, 16>, p->occ_num_sort[0][1], NB_SORT32B);
+        sort_tier(K_NUM_WARP32, k_num_sort<float, 8>, p->occ_num_sort[0][0], NB_SORT32A);
+        sort_tier(K_NUM_WARP64, k_num_sort<double, 16>, p->occ_num_sort[1][1], NB_SORT64B);
+        sort_tier(K_NUM_WARP64, k_num_sort<double, 8>, p->occ_num_sort[1][0], NB_SORT64A);
+    }
+    if (bits_tier(p, B)) {
+        // three sizes of row, so that the smaller ones leave room for more
+        // blocks: up to twice warp_max_nnz, half of block_max_nnz and all
+        const spgemm_opts& o = p->opts;
+        auto bits = [&](bool f64, int lo, int hi, int tier, int cap) {
+            launch_num_bits(p, f64, A, B, w, rptC, row_begin, colC, valC, lo, hi, tier, (cap + 3) & ~3, s);
+        };
+        if (g.bits_cap > 0) bits(false, NB_BITS32, NB_BITS32 + 1, 12, g.bits_cap);
+        bits(false, NB_BLOCK32, NB_BLOCK32 + 1, 2, o.block_max_nnz);
+        bits(true, NB_BLOCK64, NB_BLOCK64 + 1, 3, o.block_max_nnz);
+        bits(true, NB_WARP64S, NB_BLOCK64M + 1, 11, block_mid_nnz(o) > o.warp_max_nnz ? block_mid_nnz(o) : o.warp_max_nnz);
+        bits(false, NB_BLOCK32S, NB_BLOCK32M + 1, 10, block_mid_nnz(o));
+        bits(false, NB_WARP32S, NB_WARP32L + 1, 8, 2 * o.warp_max_nnz);
+    } else {
+        launch_num_hash(p, A, B, rptC, row_begin, w, colC, valC, s);
+    }
     const int PW = w.panel_cols;
     if (w.bhv && w.bpanel && B.nnz > 0)
         SPG_LAUNCH(p, K_HOT, s, k_pack_b<<<sms * 8, 256, 0, s>>>(B, w.bhot, w.bhv, w.bcv));

@@ -511,29 +511,11 @@ void occupancy_symbolic(spgemm_plan* p) {
     if (p->occ_sym_dense < 1) p->occ_sym_dense = 1;
 }
 
-void launch_symbolic(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const long long* ip,
-                     const WsPtrs& w, int* row_nnz, cudaStream_t s) {
-    GroupArgs g{};
-    g.phase = 0;
-    g.row_begin = 0;
-    g.n = A.rows;
-    g.ip = ip;
-    g.rptA = A.rpt;
-    g.row_nnz = row_nnz;
-    g.bcols = B.cols;
-    g.opts = p->opts;
-    launch_group(p, g, w, w.map, nullptr, s);
-    if (A.rows == 0) return;
+// Warp and block hash tiers: rows that outgrow the sort tier, for a B too
+// wide (or too narrow) for the bitmap tier.
+static void launch_sym_hash(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const long long* ip,
+                            const WsPtrs& w, int* row_nnz, cudaStream_t s) {
     const int sms = p->num_sms;
-    if (w.rc_slot)
-        SPG_LAUNCH(p, K_FILL, s, k_rc_reset<<<sms * 4, 256, 0, s>>>(w.rc_slot, A.rows, w.ctl));
-    SPG_LAUNCH(p, K_SYM_ESC, s, k_sym_esc<<<sms * 8, 256, 0, s>>>(A, B, w.map, w.ctl, row_nnz, SB_ESC));
-    SPG_LAUNCH(p, K_SYM_WARP, s,
-               k_sym_sort<16><<<sms * p->occ_sym_sort[1], kSortWarps * 32, 0, s>>>(
-                   A, B, w.map, w.ctl, row_nnz, SB_SORTB));
-    SPG_LAUNCH(p, K_SYM_WARP, s,
-               k_sym_sort<8><<<sms * p->occ_sym_sort[0], kSortWarps * 32, 0, s>>>(
-                   A, B, w.map, w.ctl, row_nnz, SB_SORTA));
     const size_t sw = (size_t)kWarpsPerBlockSW * kWarpTableSym * 4;
     SPG_LAUNCH(p, K_SYM_WARP, s,
                k_sym_warp<<<sms * p->occ_sym_warp, kWarpsPerBlockSW * 32, sw, s>>>(
@@ -586,6 +568,33 @@ void launch_symbolic(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, con
                    k_sym_block_staged<<<sms * p->occ_sym_staged, kStageThreads, staged_smem(), s>>>(
                        A, B, ip, w.map, w.ctl, row_nnz, staged_lo, SB_BLOCK0 + SB_BLOCK_N, 2,
                        hash_load(p)));
+}
+
+void launch_symbolic(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const long long* ip,
+                     const WsPtrs& w, int* row_nnz, cudaStream_t s) {
+    GroupArgs g{};
+    g.phase = 0;
+    g.row_begin = 0;
+    g.n = A.rows;
+    g.ip = ip;
+    g.rptA = A.rpt;
+    g.row_nnz = row_nnz;
+    g.bcols = B.cols;
+    g.opts = p->opts;
+    launch_group(p, g, w, w.map, nullptr, s);
+    if (A.rows == 0) return;
+    const int sms = p->num_sms;
+    if (w.rc_slot)
+        SPG_LAUNCH(p, K_FILL, s, k_rc_reset<<<sms * 4, 256, 0, s>>>(w.rc_slot, A.rows, w.ctl));
+    SPG_LAUNCH(p, K_SYM_ESC, s, k_sym_esc<<<sms * 8, 256, 0, s>>>(A, B, w.map, w.ctl, row_nnz, SB_ESC));
+    SPG_LAUNCH(p, K_SYM_WARP, s,
+               k_sym_sort<16><<<sms * p->occ_sym_sort[1], kSortWarps * 32, 0, s>>>(
+                   A, B, w.map, w.ctl, row_nnz, SB_SORTB));
+    SPG_LAUNCH(p, K_SYM_WARP, s,
+               k_sym_sort<8><<<sms * p->occ_sym_sort[0], kSortWarps * 32, 0, s>>>(
+                   A, B, w.map, w.ctl, row_nnz, SB_SORTA));
+    if (bits_tier(p, B)) launch_sym_bits(p, A, B, w, row_nnz, SB_WARP, SB_BLOCK0 + SB_BLOCK_N, 0, s);
+    else launch_sym_hash(p, A, B, ip, w, row_nnz, s);
     if (B.cols <= kNarrowCols)
         SPG_LAUNCH(p, K_SYM_NARROW, s,
                    k_sym_narrow<<<sms * (64 / narrow_warps(p) > 1 ? 64 / narrow_warps(p) : 1),

@@ -1,0 +1,43 @@
+"""Bitmap tiers at the edges of their tiles, row classes and column limits,
+against the oracle: A rows around the tile sizes, few and many products an
+entry, rows of a handful to nearly all columns, fp32 and fp64 rows, repeated
+and unsorted columns in B."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2512_12036_gb300 import DeviceCSR, Plan, gen
+from parity import compare
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("cols", [1025, 4097, 40_000, 131_071, 1 << 19, (1 << 19) + 1])
+@pytest.mark.parametrize("messy", [False, True])
+def test_rows_at_tile_and_class_edges(cols, messy):
+    rng = np.random.default_rng(cols + messy)
+    lens = np.concatenate([np.full(1500, 24), np.full(300, 0), np.full(40, min(cols, 900))])
+    r = np.repeat(np.arange(lens.size), lens)
+    c = np.concatenate([rng.choice(cols, size=n, replace=False) for n in lens])
+    c[0], c[-1] = cols - 1, 0
+    if messy:                                     # repeated columns, rows out of order
+        r, c = np.concatenate([r, r[::7]]), np.concatenate([c, c[::7]])
+        p = np.lexsort((rng.random(r.size), r))
+        r, c = r[p], c[p]
+    B = gen.csr_from_coo(lens.size, cols, r, c, gen.uniform_open_closed(rng, r.size), sort=not messy)
+    ra, ca = [], []
+    for na in [30, 60, 127, 128, 129, 167, 168, 255, 256, 257, 511, 512, 513, 1100]:
+        for long_rows in (0, 1, 12, 40):          # 24 to 60,000 products a row
+            k = rng.choice(1800, size=na, replace=False)
+            k[:min(long_rows, na)] = 1800 + rng.choice(40, size=min(long_rows, na), replace=False)
+            ra.append(np.full(na, len(ra)))
+            ca.append(rng.permutation(k))
+    A = gen.csr_from_coo(len(ra), lens.size, np.concatenate(ra), np.concatenate(ca),
+                         gen.uniform_open_closed(rng, sum(x.size for x in ra)), sort=False)
+    ref = oracle.spgemm(A, B)
+    dA, dB = DeviceCSR.from_host(A), DeviceCSR.from_host(B)
+    for opts in ({}, {"warp_max_nnz": 100, "block_max_nnz": 2000}):
+        C = Plan(**opts).spgemm(dA, dB)
+        torch.cuda.synchronize()
+        compare(C.to_host(), ref)
