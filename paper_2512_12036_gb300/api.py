@@ -119,12 +119,15 @@ class Plan:
 
     def workspace(self, A: DeviceCSR, B: DeviceCSR, stream=None) -> torch.Tensor:
         """A 256-byte aligned, initialised workspace for operands of these shapes."""
+        ws = self._workspace_buffer(A, B)
+        self.workspace_init(ws, stream)
+        return ws
+
+    def _workspace_buffer(self, A: DeviceCSR, B: DeviceCSR) -> torch.Tensor:
         nbytes = self.workspace_bytes(A, B)
         ws = torch.empty(nbytes + 256, dtype=torch.uint8, device=A.device)
         off = (-ws.data_ptr()) % 256
-        ws = ws[off:off + nbytes]
-        self.workspace_init(ws, stream)
-        return ws
+        return ws[off:off + nbytes]
 
     def workspace_init(self, ws: torch.Tensor, stream=None) -> None:
         check(_lib.lib().spgemm_workspace_init(self.handle, _ptr(ws), ws.numel(), _stream(stream)),
@@ -285,7 +288,7 @@ class Plan:
         ``ip_row`` (int64, A.rows, on the device) receives the per-row
         intermediate-product counts of the call (Algorithm 1) when given."""
         if ws is None:
-            ws = self.workspace(A, B)
+            ws = self._workspace_buffer(A, B)      # (the call initialises it)
         dev = A.device
         if ip_row is None:
             ip_row = torch.empty(A.rows, dtype=torch.int64, device=dev)

@@ -22,6 +22,7 @@ class SpGEMMFunction(torch.autograd.Function):
         ctx.plan = plan
         ctx.A, ctx.B, ctx.C = Av, Bv, C
         ctx.mark_non_differentiable(C.row_ptr, C.col)
+        ctx.set_materialize_grads(False)          # no zeros for the index outputs
         return C.row_ptr, C.col, C.val
 
     @staticmethod

@@ -9,6 +9,7 @@ namespace spg {
 void occupancy_symbolic(spgemm_plan* p);
 void occupancy_numeric(spgemm_plan* p);
 void occupancy_bits(spgemm_plan* p);
+void occupancy_narrow(spgemm_plan* p);
 void occupancy_backward(spgemm_plan* p);
 void occupancy_mcl(spgemm_plan* p);
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -50,6 +51,12 @@ WsLayout ws_layout(const spgemm_plan* p, long long m, long long b_rows, long lon
         off = align256(off + 8 * (size_t)b_nnz);
     }
     const long long wpr = (b_cols + 31) / 32;
+    if (b_nnz > 0 && wpr > 0 && b_cols <= kNarrowCols && m > 0) {
+        L.nb_bits = off;
+        off = align256(off + sizeof(unsigned) * (size_t)wpr * (size_t)b_rows);
+        L.nc_bits = off;
+        off = align256(off + sizeof(unsigned) * (size_t)wpr * (size_t)m);
+    }
     if (p->opts.row_cache_mb > 0 && m > 0 && wpr > 0 && wpr <= kRowCacheMaxWords) {
         const size_t bytes = (size_t)p->opts.row_cache_mb << 20;
         // per slot: the bitmap, and the entry count of each table panel
@@ -95,6 +102,8 @@ WsPtrs ws_ptrs(const WsLayout& L, void* ws, int panel_cols) {
     w.rc_pc = L.rc_nslots > 0 && L.rc_pc > 0 ? (int*)(b + L.rc_pc) : nullptr;
     w.rc_nslots = L.rc_nslots;
     w.rc_wpr = L.rc_wpr;
+    w.nb_bits = L.nc_bits > 0 ? (unsigned*)(b + L.nb_bits) : nullptr;
+    w.nc_bits = L.nc_bits > 0 ? (unsigned*)(b + L.nc_bits) : nullptr;
     w.nblk = L.nblk;
     w.nscan = L.nscan;
     w.panels = L.panels;
@@ -114,6 +123,7 @@ void init_occupancy(spgemm_plan* p) {
     occupancy_symbolic(p);
     occupancy_numeric(p);
     occupancy_bits(p);
+    occupancy_narrow(p);
     occupancy_backward(p);
     occupancy_mcl(p);
 }
@@ -209,20 +219,26 @@ static int map_status(int bits) {
     return SPGEMM_OK;
 }
 
-// Synchronise, fetch totals[which] (if out) and the status word, clear it.
-static int sync_read(Ctl* ctl, int which, int64_t* out, cudaStream_t s) {
-    Ctl h;                                   // its head, up to and including the totals
-    cudaError_t e = cudaMemcpyAsync(&h, ctl, offsetof(Ctl, totals) + sizeof(h.totals),
-                                    cudaMemcpyDeviceToHost, s);
+// Synchronise, fetch the control block up to `bytes` and the status word (the
+// return value), clear it.
+static int sync_ctl(Ctl* ctl, Ctl* h, size_t bytes, cudaStream_t s) {
+    cudaError_t e = cudaMemcpyAsync(h, ctl, bytes, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) return SPGEMM_ERR_CUDA;
-    if (out && which >= 0) *out = h.totals[which];
-    if (h.status) {
+    if (h->status) {
         int zero = 0;
         cudaMemcpyAsync(&ctl->status, &zero, sizeof(int), cudaMemcpyHostToDevice, s);
         cudaStreamSynchronize(s);
     }
-    return map_status(h.status);
+    return map_status(h->status);
+}
+
+// The same for totals[which] (if out).
+static int sync_read(Ctl* ctl, int which, int64_t* out, cudaStream_t s) {
+    Ctl h;                                   // its head, up to and including the totals
+    const int rc = sync_ctl(ctl, &h, offsetof(Ctl, totals) + sizeof(h.totals), s);
+    if (rc != SPGEMM_ERR_CUDA && out && which >= 0) *out = h.totals[which];
+    return rc;
 }
 
 extern "C" {
@@ -429,8 +445,8 @@ int spgemm_symbolic(const spgemm_plan* plan, const spgemm_csr* A, const spgemm_c
     WsPtrs w = ws_ptrs(L, ws, plan->opts.panel_cols);
     CsrDev dA = dev_view(A), dB = dev_view(B);
     launch_symbolic(plan, dA, dB, (const long long*)ip_row, w, row_nnz, s);
-    launch_bpanel(plan, dB, w, s);
-    launch_hot(plan, dB, w, s);
+    launch_dense_tables(plan, dB, w, s);
+    if (dB.cols <= plan->opts.block_max_nnz) launch_check_rpt(plan, dB, w, s);   // (as the tables do)
     launch_nnz_total(plan, row_nnz, A->rows, w, s);
     rc = cuda_err(cudaGetLastError());
     if (rc) return rc;
@@ -478,23 +494,39 @@ int spgemm(const spgemm_plan* plan, const spgemm_csr* A, const spgemm_csr* B, vo
     if (!alloc || !nnz_C || !row_ptr_C) return SPGEMM_ERR_INVALID;
     rc = spgemm_workspace_init(plan, ws, ws_bytes, stream);
     if (rc) return rc;
-    rc = spgemm_count(plan, A, B, ws, ws_bytes, ip_row, nullptr, stream);
+    if (A->rows > 0 && (!ip_row || !row_nnz)) return SPGEMM_ERR_INVALID;
+    WsLayout L;
+    rc = check_ws(plan, A, B, ws, ws_bytes, &L);
     if (rc) return rc;
-    int64_t total = 0;
-    rc = spgemm_symbolic(plan, A, B, ip_row, ws, ws_bytes, row_nnz, &total, stream);
+    cudaStream_t s = (cudaStream_t)stream;
+    WsPtrs w = ws_ptrs(L, ws, plan->opts.panel_cols);
+    const CsrDev dA = dev_view(A), dB = dev_view(B);
+    const long long* ip = (const long long*)ip_row;
+    launch_ip_count(plan, dA, dB, (long long*)ip_row, w, s);
+    launch_symbolic(plan, dA, dB, ip, w, row_nnz, s);
+    launch_row_ptr(plan, row_nnz, A->rows, w, row_ptr_C, s);
+    // the accumulation phase's grouping before the wait for the size of C: the
+    // host then knows which tiers have rows, launches only those, and builds
+    // the dense tiers' tables of B only for them (a 4,096-vertex product made
+    // 52 launches, 12 now)
+    launch_numeric_group(plan, dA, dB, ip, 0, A->rows, row_ptr_C, w, s);
+    rc = cuda_err(cudaGetLastError());
     if (rc) return rc;
+    Ctl h;
+    rc = sync_ctl(w.ctl, &h, sizeof(Ctl), s);
+    if (rc && rc != SPGEMM_ERR_OVERFLOW) return rc;
+    const int64_t total = h.totals[2];
     *nnz_C = total;
     if (total > 2147483647ll) return SPGEMM_ERR_OVERFLOW;
-    rc = spgemm_row_ptr(plan, row_nnz, A->rows, ws, ws_bytes, row_ptr_C, nullptr, stream);
     if (rc) return rc;
     int32_t* col = nullptr;
     float* val = nullptr;
     if (alloc(alloc_ctx, total, &col, &val) != 0) return SPGEMM_ERR_BUDGET;
     if (total > 0 && (!col || !val)) return SPGEMM_ERR_BUDGET;
-    rc = spgemm_numeric(plan, A, B, ip_row, 0, A->rows, row_ptr_C, ws, ws_bytes, col, val, stream);
+    launch_numeric_tiers(plan, dA, dB, 0, A->rows, row_ptr_C, w, col, val, h.bin_off, s);
+    rc = cuda_err(cudaGetLastError());
     if (rc) return rc;
-    WsLayout L = ws_layout(plan, A->rows, B->rows, B->cols, B->nnz);
-    return sync_read(ws_ptrs(L, ws, plan->opts.panel_cols).ctl, -1, nullptr, (cudaStream_t)stream);
+    return sync_read(w.ctl, -1, nullptr, s);
 }
 
 int spgemm_batched(const spgemm_plan* plan, const spgemm_csr* A, const spgemm_csr* B, void* ws,
@@ -514,8 +546,7 @@ int spgemm_batched(const spgemm_plan* plan, const spgemm_csr* A, const spgemm_cs
     CsrDev dA = dev_view(A), dB = dev_view(B);
     launch_ip_count(plan, dA, dB, (long long*)ip_row, w, s);
     launch_symbolic(plan, dA, dB, (const long long*)ip_row, w, row_nnz, s);
-    launch_bpanel(plan, dB, w, s);
-    launch_hot(plan, dB, w, s);
+    launch_dense_tables(plan, dB, w, s);
     launch_row_ptr(plan, row_nnz, A->rows, w, row_ptr_C, s);
     launch_copy_total(plan, w, 2, (long long*)nnz_C, s);
     launch_numeric(plan, dA, dB, (const long long*)ip_row, 0, A->rows, row_ptr_C, w, col_C, val_C,

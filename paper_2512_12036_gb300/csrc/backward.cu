@@ -32,10 +32,22 @@ struct BwdArgs {
     int P, PW;
 };
 
-__global__ void k_bwd_zero(double* p, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        p[i] = 0.0;
+// Before the tiers: both gradients cleared (A entries of a row whose row of C
+// is empty are never visited: no product, gradient 0) and B's row pointers
+// checked.
+__global__ void k_bwd_prep(CsrDev B, double* dB64, float* dA, long long a_nnz, Ctl* ctl) {
+    const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long step = (long long)gridDim.x * blockDim.x;
+    if (dB64)
+        for (long long i = i0; i < B.nnz; i += step) dB64[i] = 0.0;
+    if (dA)
+        for (long long i = i0; i < a_nnz; i += step) dA[i] = 0.f;
+    bool bad = false;
+    for (long long i = i0; i < B.rows; i += step) {
+        const int s = B.rpt[i], e = B.rpt[i + 1];
+        bad |= s < 0 || e < s || (long long)e > B.nnz;
+    }
+    if (bad) set_status(ctl, ST_INVALID);
 }
 
 __global__ void k_bwd_convert(const double* src, float* dst, long long n) {
@@ -398,13 +410,11 @@ void launch_backward(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, con
     const int sms = p->num_sms;
     BwdArgs x{A, B, rptC, colC, dC, dA, dB ? dB64 : nullptr, w.ctl, w.map, nullptr, w.panels,
               w.panel_cols};
-    if (dB && B.nnz > 0)
-        SPG_LAUNCH(p, K_BWD, s, k_bwd_zero<<<sms * 4, 256, 0, s>>>(dB64, B.nnz));
-    // rows whose C row is empty are never visited: their A entries have no
-    // product, so their gradient is 0
-    if (dA && A.nnz > 0) cudaMemsetAsync(dA, 0, sizeof(float) * (size_t)A.nnz, s);
-    // the heavy tier needs B's panel table (built into this workspace)
-    launch_bpanel(p, B, w, s);
+    SPG_LAUNCH(p, K_BWD, s, k_bwd_prep<<<sms * 8, 256, 0, s>>>(B, dB ? dB64 : nullptr, dA, A.nnz, w.ctl));
+    // the panel tier needs B's panel table (built into this workspace); with
+    // few columns every row of C is in the dense tier
+    const bool few = B.cols <= kBwdDenseCols;
+    if (!few) launch_bpanel(p, B, w, s);
     x.tab = w.bpanel;
     GroupArgs g{};
     g.phase = 3;
@@ -421,20 +431,21 @@ void launch_backward(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, con
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, kBwdWarps * 32, smem);
             return sms * (occ > 0 ? occ : 1);
         };
-        if (B.cols <= kBwdDenseCols) {
+        if (few) {
             const size_t sd = (size_t)kBwdWarps * B.cols * 4;
             SPG_LAUNCH(p, K_BWD, s,
                        k_bwd_dense<<<resident((const void*)k_bwd_dense, sd), kBwdWarps * 32, sd, s>>>(
                            x, BW_DENSE));
+        } else {
+            const size_t sw = (size_t)kBwdWarps * kBwdWarpSlots * 8;
+            SPG_LAUNCH(p, K_BWD, s,
+                       k_bwd_warp<<<resident((const void*)k_bwd_warp, sw), kBwdWarps * 32, sw, s>>>(
+                           x, BW_WARP));
+            SPG_LAUNCH(p, K_BWD, s,
+                       k_bwd_block<<<sms, kBwdBlockThreads, kBwdBlockSlots * 8, s>>>(x, BW_BLOCK, 6));
+            SPG_LAUNCH(p, K_BWD, s,
+                       k_bwd_panel<<<sms, kBwdBlockThreads, kBwdPanel * 4, s>>>(x, BW_PANEL, 7, dA64));
         }
-        const size_t sw = (size_t)kBwdWarps * kBwdWarpSlots * 8;
-        SPG_LAUNCH(p, K_BWD, s,
-                   k_bwd_warp<<<resident((const void*)k_bwd_warp, sw), kBwdWarps * 32, sw, s>>>(
-                       x, BW_WARP));
-        SPG_LAUNCH(p, K_BWD, s,
-                   k_bwd_block<<<sms, kBwdBlockThreads, kBwdBlockSlots * 8, s>>>(x, BW_BLOCK, 6));
-        SPG_LAUNCH(p, K_BWD, s,
-                   k_bwd_panel<<<sms, kBwdBlockThreads, kBwdPanel * 4, s>>>(x, BW_PANEL, 7, dA64));
     }
     if (dB && B.nnz > 0)
         SPG_LAUNCH(p, K_BWD, s, k_bwd_convert<<<sms * 4, 256, 0, s>>>(dB64, dB, B.nnz));

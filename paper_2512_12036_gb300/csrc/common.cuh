@@ -33,11 +33,12 @@ struct Ctl {
                                 // more A entries than the rank-compacted kernel takes
     int dense_uncached;         // accumulation grouping: a row of the fp64-bound dense tier
                                 // has no cached bitmap
-    int pad0;
+    int narrow_dup;             // a row of a narrow B may repeat a column
     long long totals[8];        // 0: IP total, 1: nnz total, 2: scan total
     int work[kMaxTiers];        // dynamic row counters of the block-per-row tiers
     int bin_off[kNumBins + 1];  // start of every bin in the row map
-    int pad1[256 - 6 - 16 - kMaxTiers - (kNumBins + 1)];
+    int bin_rows[kNumBins];     // rows of every bin (grouping)
+    int pad1[256 - 6 - 16 - kMaxTiers - (kNumBins + 1) - kNumBins];
 };
 static_assert(sizeof(Ctl) % 256 == 0, "Ctl must keep the following arrays aligned");
 

@@ -8,19 +8,6 @@ namespace spg {
 // Small utilities
 // ---------------------------------------------------------------------------
 
-__global__ void k_fill_i64(long long* p, long long n, long long v) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
-         i += (long long)gridDim.x * blockDim.x)
-        p[i] = v;
-}
-
-void launch_fill_i64(const spgemm_plan* pl, long long* p, long long n, long long v, cudaStream_t s) {
-    if (n <= 0) return;
-    long long blocks = (n + 255) / 256;
-    if (blocks > 4096) blocks = 4096;
-    SPG_LAUNCH(pl, K_FILL, s, k_fill_i64<<<(int)blocks, 256, 0, s>>>(p, n, v));
-}
-
 template <typename T>
 __global__ void k_sum_to(const T* x, long long n, long long* out) {
     __shared__ long long red[33];
@@ -33,15 +20,6 @@ __global__ void k_sum_to(const T* x, long long n, long long* out) {
 }
 
 __global__ void k_zero_total(Ctl* ctl, int which) { ctl->totals[which] = 0; }
-
-// Row pointers must be monotone and inside [0, nnz].
-__global__ void k_check_rpt(CsrDev M, Ctl* ctl) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < M.rows;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int s = M.rpt[i], e = M.rpt[i + 1];
-        if (s < 0 || e < s || (long long)e > M.nnz) set_status(ctl, ST_INVALID);
-    }
-}
 
 // ---------------------------------------------------------------------------
 // Algorithm 1, balanced over nonzeros: each block takes a tile of A's stored
@@ -67,6 +45,7 @@ __device__ __forceinline__ int row_of(const int* rpt, long long j, int lo, int h
 __global__ void __launch_bounds__(kCountThreads) k_ip_count(CsrDev A, CsrDev B, long long* ip,
                                                             Ctl* ctl) {
     __shared__ int s_r0, s_r1;
+    __shared__ long long red[33];
     const int m = A.rows;
     const long long J0 = A.rpt[0], J1 = A.rpt[m];
     if (J0 < 0 || J1 < J0 || J1 > A.nnz) {
@@ -84,6 +63,7 @@ __global__ void __launch_bounds__(kCountThreads) k_ip_count(CsrDev A, CsrDev B, 
     __syncthreads();
     const int r0 = s_r0, r1 = s_r1;
     const int lane = lane_id();
+    long long sum = 0;                               // this thread's products
     for (int it = 0; it < kCountItems; ++it) {
         const long long j = jb + (long long)it * kCountThreads + threadIdx.x;
         int row = -1;
@@ -93,6 +73,7 @@ __global__ void __launch_bounds__(kCountThreads) k_ip_count(CsrDev A, CsrDev B, 
             int bs, len;
             a_entry(A, B, (int)j, bs, len, ctl);
             v = len;
+            sum += len;
         }
         // segmented inclusive scan over contiguous equal rows
 #pragma unroll
@@ -105,26 +86,54 @@ __global__ void __launch_bounds__(kCountThreads) k_ip_count(CsrDev A, CsrDev B, 
         const bool last = (lane == 31) || rn != row;
         if (last && row >= 0 && v != 0) atomicAdd((unsigned long long*)&ip[row], (unsigned long long)v);
     }
+    sum = block_sum(sum, red);
+    if (threadIdx.x == 0 && sum != 0) atomicAdd((unsigned long long*)&ctl->totals[0], (unsigned long long)sum);
+}
+
+// One pass over the rows before the count: zero counts, both operands' row
+// pointers checked, the total reset.
+__global__ void k_count_prep(CsrDev A, CsrDev B, long long* ip, Ctl* ctl) {
+    const long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const long long step = (long long)gridDim.x * blockDim.x;
+    if (i0 == 0) ctl->totals[0] = 0;
+    bool bad = false;
+    for (long long i = i0; i < A.rows; i += step) {
+        const int s = A.rpt[i], e = A.rpt[i + 1];
+        bad |= s < 0 || e < s || (long long)e > A.nnz;
+        ip[i] = 0;
+    }
+    for (long long i = i0; i < B.rows; i += step) {
+        const int s = B.rpt[i], e = B.rpt[i + 1];
+        bad |= s < 0 || e < s || (long long)e > B.nnz;
+    }
+    if (bad) set_status(ctl, ST_INVALID);
+}
+
+// Row pointers must be monotone and inside [0, nnz].
+__global__ void k_check_rpt(CsrDev M, Ctl* ctl) {
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < M.rows;
+         i += (long long)gridDim.x * blockDim.x) {
+        const int s = M.rpt[i], e = M.rpt[i + 1];
+        if (s < 0 || e < s || (long long)e > M.nnz) set_status(ctl, ST_INVALID);
+    }
+}
+
+void launch_check_rpt(const spgemm_plan* p, const CsrDev& M, const WsPtrs& w, cudaStream_t s) {
+    if (M.rows == 0) return;
+    const int blocks = (M.rows + 255) / 256 < 4096 ? (M.rows + 255) / 256 : 4096;
+    SPG_LAUNCH(p, K_CHECK_RPT, s, k_check_rpt<<<blocks, 256, 0, s>>>(M, w.ctl));
 }
 
 void launch_ip_count(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, long long* ip,
                      const WsPtrs& w, cudaStream_t s) {
     if (A.rows == 0) return;
-    launch_fill_i64(p, ip, A.rows, 0, s);
-    {
-        const int blocks = (int)((A.rows + 255) / 256 < 4096 ? (A.rows + 255) / 256 : 4096);
-        SPG_LAUNCH(p, K_CHECK_RPT, s, k_check_rpt<<<blocks, 256, 0, s>>>(A, w.ctl));
-    }
-    if (B.rows > 0) {
-        const int blocks = (int)((B.rows + 255) / 256 < 4096 ? (B.rows + 255) / 256 : 4096);
-        SPG_LAUNCH(p, K_CHECK_RPT, s, k_check_rpt<<<blocks, 256, 0, s>>>(B, w.ctl));
-    }
-    SPG_LAUNCH(p, K_ZERO, s, k_zero_total<<<1, 1, 0, s>>>(w.ctl, 0));
+    const int rows = A.rows > B.rows ? A.rows : B.rows;
+    const int blocks = (rows + 255) / 256 < 4096 ? (rows + 255) / 256 : 4096;
+    SPG_LAUNCH(p, K_CHECK_RPT, s, k_count_prep<<<blocks, 256, 0, s>>>(A, B, ip, w.ctl));
     if (A.nnz > 0) {
         const long long tiles = (A.nnz + kCountTile - 1) / kCountTile;
         SPG_LAUNCH(p, K_IP_COUNT, s, k_ip_count<<<(unsigned)tiles, kCountThreads, 0, s>>>(A, B, ip, w.ctl));
     }
-    SPG_LAUNCH(p, K_SUM, s, k_sum_to<long long><<<256, 256, 0, s>>>(ip, A.rows, &w.ctl->totals[0]));
 }
 
 void launch_nnz_total(const spgemm_plan* p, const int* row_nnz, int n, const WsPtrs& w, cudaStream_t s) {
@@ -214,58 +223,83 @@ __global__ void __launch_bounds__(kBinRows) k_group_hist(GroupArgs g, int nblk, 
     if (threadIdx.x < kNumBins) blk_counts[threadIdx.x * nblk + blockIdx.x] = hist[threadIdx.x];
 }
 
-// One block: exclusive scan of the (bin-major) block counts in place; bin
-// starts into ctl->bin_off (and offsets_out for the public grouping call).
-__global__ void __launch_bounds__(1024) k_group_scan(int nblk, int* blk_counts, Ctl* ctl,
-                                                     int* offsets_out, int ngroups) {
+// A block per bin: exclusive scan of the bin's block counts in place and the
+// bin's rows into ctl->bin_rows (one block over all 64 bins was a chain of 72
+// barriers for 1,150 row blocks, 27 us; under 3 us now).
+constexpr int kGroupScanThreads = 256;
+
+__global__ void __launch_bounds__(kGroupScanThreads) k_group_scan(int nblk, int* blk_counts, Ctl* ctl) {
     __shared__ int scratch[33];
-    const long long total_n = (long long)kNumBins * nblk;
+    int* counts = blk_counts + (long long)blockIdx.x * nblk;
     int carry = 0;
-    for (long long base = 0; base < total_n; base += blockDim.x) {
-        const long long i = base + threadIdx.x;
-        const int v = i < total_n ? blk_counts[i] : 0;
+    for (int base = 0; base < nblk; base += kGroupScanThreads) {
+        const int i = base + threadIdx.x;
+        const int v = i < nblk ? counts[i] : 0;
         int tot;
         const int ex = block_excl_scan(v, scratch, &tot);
-        if (i < total_n) blk_counts[i] = carry + ex;
+        if (i < nblk) counts[i] = carry + ex;
         carry += tot;
     }
-    __syncthreads();
-    if (threadIdx.x <= kNumBins) {
-        const int b = threadIdx.x;
-        int off;
-        if (b == kNumBins) off = carry;
-        else off = nblk > 0 ? blk_counts[(long long)b * nblk] : 0;
-        ctl->bin_off[b] = off;
-        if (offsets_out && b <= ngroups) offsets_out[b] = b == ngroups ? carry : off;
+    if (threadIdx.x == 0) ctl->bin_rows[blockIdx.x] = carry;
+    // (the scatter, which follows, sets the flags)
+    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->dense_wide = ctl->dense_uncached = 0;
+}
+
+// Bin starts from the bins' row counts, by one warp: base[b] for every bin in
+// shared memory and, from one block of the launch, ctl->bin_off (offsets_out
+// for the public grouping call) and the tiers' row counters.
+__device__ __forceinline__ void group_bases(const int* rows, int* base, bool write, Ctl* ctl,
+                                            int* offsets_out, int ngroups) {
+    const int lane = lane_id();
+    const int a = rows[2 * lane], b = rows[2 * lane + 1];
+    const int incl = warp_incl_scan(a + b), ex = incl - a - b;
+    base[2 * lane] = ex;
+    base[2 * lane + 1] = ex + a;
+    if (!write) return;
+    ctl->bin_off[2 * lane] = ex;
+    ctl->bin_off[2 * lane + 1] = ex + a;
+    if (lane == 31) ctl->bin_off[kNumBins] = incl;
+    if (lane < kMaxTiers) ctl->work[lane] = 0;
+    if (offsets_out) {
+        const int total = __shfl_sync(kFull, incl, 31);
+        for (int q = 0; q < 2; ++q) {
+            const int g = 2 * lane + q;
+            if (g <= ngroups) offsets_out[g] = g == ngroups ? total : (q ? ex + a : ex);
+        }
     }
-    if (threadIdx.x < kMaxTiers) ctl->work[threadIdx.x] = 0;
-    if (threadIdx.x == 0) {
-        ctl->dense_wide = 0;
-        ctl->dense_uncached = 0;
+}
+
+// accumulation: flag an fp32 dense row too wide for the rank-compacted
+// kernel, so the fallback kernel runs only when it has rows, and an
+// fp64-bound dense row without a cached bitmap, so the kernel for those runs
+// only when there are some
+__device__ __forceinline__ void group_flags(const GroupArgs& g, int r, int b, Ctl* ctl) {
+    if (g.phase != 1 || b < 0) return;
+    // (no tier is launched for rows of more entries than B has columns)
+    if (g.rptC[r + 1] - g.rptC[r] > g.bcols) set_status(ctl, ST_INTERNAL);
+    if (b >= NB_DENSE32_0 && b < NB_DENSE32_0 + NB_DENSE_N) {
+        const int row = g.row_begin + r;
+        if (g.rptA[row + 1] - g.rptA[row] > kRankTileEntries) ctl->dense_wide = 1;
     }
+    if (b >= NB_DENSE64_0 && b < NB_DENSE64_0 + NB_DENSE_N &&
+        (g.rc_slot == nullptr || g.rc_slot[g.row_begin + r] < 0))
+        ctl->dense_uncached = 1;
 }
 
 __global__ void __launch_bounds__(kBinRows) k_group_scatter(GroupArgs g, int nblk,
                                                             const int* blk_counts, int* map,
-                                                            Ctl* ctl) {
+                                                            Ctl* ctl, int* offsets_out,
+                                                            int ngroups) {
     __shared__ int wcount[kBinRows / 32][kNumBins];
-    const int warp = threadIdx.x >> 5, lane = lane_id();
+    __shared__ int base[kNumBins];
+    const int warp = threadIdx.x >> 5;
+    if (warp == 0) group_bases(ctl->bin_rows, base, blockIdx.x == 0, ctl, offsets_out, ngroups);
     for (int i = threadIdx.x; i < (kBinRows / 32) * kNumBins; i += blockDim.x)
         (&wcount[0][0])[i] = 0;
     __syncthreads();
     const int r = blockIdx.x * kBinRows + threadIdx.x;
     const int b = r < g.n ? bin_of(g, r, false) : -1;
-    // accumulation: flag an fp32 dense row too wide for the rank-compacted
-    // kernel, so the fallback kernel runs only when it has rows
-    // and an fp64-bound dense row without a cached bitmap, so the kernel
-    // for those runs only when there are some
-    if (g.phase == 1 && b >= NB_DENSE32_0 && b < NB_DENSE32_0 + NB_DENSE_N) {
-        const int row = g.row_begin + r;
-        if (g.rptA[row + 1] - g.rptA[row] > kRankTileEntries) ctl->dense_wide = 1;
-    }
-    if (g.phase == 1 && b >= NB_DENSE64_0 && b < NB_DENSE64_0 + NB_DENSE_N &&
-        (g.rc_slot == nullptr || g.rc_slot[g.row_begin + r] < 0))
-        ctl->dense_uncached = 1;
+    group_flags(g, r, b, ctl);
     const unsigned peers = __match_any_sync(kFull, b);
     const int rank = __popc(peers & lanemask_lt());
     if (b >= 0 && rank == 0) wcount[warp][b] = __popc(peers);
@@ -279,20 +313,78 @@ __global__ void __launch_bounds__(kBinRows) k_group_scatter(GroupArgs g, int nbl
         }
     }
     __syncthreads();
-    if (b >= 0) map[blk_counts[(long long)b * nblk + blockIdx.x] + wcount[warp][b] + rank] = r;
+    if (b >= 0) map[base[b] + blk_counts[(long long)b * nblk + blockIdx.x] + wcount[warp][b] + rank] = r;
+}
+
+// The whole grouping of up to kGroupSmallRows rows in one block, thread t
+// taking rows t, t + 1024, ...: one launch instead of three, which is what a
+// small product waits for. Same map: rows of a bin in ascending order.
+constexpr int kGroupSmallRows = 8 * kBinRows;
+
+__global__ void __launch_bounds__(kBinRows) k_group_small(GroupArgs g, int* map, Ctl* ctl,
+                                                          int* offsets_out, int ngroups) {
+    constexpr int kChunks = kGroupSmallRows / kBinRows;
+    __shared__ int wcount[kBinRows / 32][kNumBins];
+    __shared__ int base[kNumBins], total[kNumBins];
+    const int t = threadIdx.x, warp = t >> 5;
+    int bins[kChunks];
+    if (t < kNumBins) total[t] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < kChunks; ++c) {
+        const int r = c * kBinRows + t;
+        bins[c] = -1;
+        if (c * kBinRows < g.n) {                     // block-uniform
+            if (r < g.n) bins[c] = bin_of(g, r, true);
+            const unsigned peers = __match_any_sync(kFull, bins[c]);
+            if (bins[c] >= 0 && (peers & lanemask_lt()) == 0) atomicAdd(&total[bins[c]], __popc(peers));
+        }
+    }
+    __syncthreads();
+    if (warp == 0) group_bases(total, base, true, ctl, offsets_out, ngroups);
+    if (t == 32) ctl->dense_wide = ctl->dense_uncached = 0;
+    __syncthreads();                                 // (flags are reset before they are set)
+#pragma unroll
+    for (int c = 0; c < kChunks; ++c) {
+        if (c * kBinRows >= g.n) break;              // block-uniform
+        for (int i = t; i < (kBinRows / 32) * kNumBins; i += kBinRows) (&wcount[0][0])[i] = 0;
+        __syncthreads();
+        const int r = c * kBinRows + t, b = bins[c];
+        group_flags(g, r, b, ctl);
+        const unsigned peers = __match_any_sync(kFull, b);
+        const int rank = __popc(peers & lanemask_lt());
+        if (b >= 0 && rank == 0) wcount[warp][b] = __popc(peers);
+        __syncthreads();
+        if (t < kNumBins) {
+            int acc = base[t];
+            for (int w = 0; w < kBinRows / 32; ++w) {
+                const int n = wcount[w][t];
+                wcount[w][t] = acc;
+                acc += n;
+            }
+            base[t] = acc;
+        }
+        __syncthreads();
+        if (b >= 0) map[wcount[warp][b] + rank] = r;
+        __syncthreads();
+    }
 }
 
 void launch_group(const spgemm_plan* p, const GroupArgs& g, const WsPtrs& w, int* map_out,
                   int* offsets_out, cudaStream_t s) {
     const int nblk = (g.n + kBinRows - 1) / kBinRows;
-    if (nblk > 0)
-        SPG_LAUNCH(p, K_GROUP_HIST, s, k_group_hist<<<nblk, kBinRows, 0, s>>>(g, nblk, w.blk_counts));
-    SPG_LAUNCH(p, K_GROUP_SCAN, s,
-               k_group_scan<<<1, 1024, 0, s>>>(nblk, w.blk_counts, w.ctl, offsets_out,
-                                               g.phase == 2 ? g.nthr + 1 : 0));
-    if (nblk > 0)
+    if (g.n <= kGroupSmallRows) {
         SPG_LAUNCH(p, K_GROUP_SCATTER, s,
-                   k_group_scatter<<<nblk, kBinRows, 0, s>>>(g, nblk, w.blk_counts, map_out, w.ctl));
+                   k_group_small<<<1, kBinRows, 0, s>>>(g, map_out, w.ctl, offsets_out,
+                                                        g.phase == 2 ? g.nthr + 1 : 0));
+        return;
+    }
+    SPG_LAUNCH(p, K_GROUP_HIST, s, k_group_hist<<<nblk, kBinRows, 0, s>>>(g, nblk, w.blk_counts));
+    SPG_LAUNCH(p, K_GROUP_SCAN, s,
+               k_group_scan<<<kNumBins, kGroupScanThreads, 0, s>>>(nblk, w.blk_counts, w.ctl));
+    SPG_LAUNCH(p, K_GROUP_SCATTER, s,
+               k_group_scatter<<<nblk, kBinRows, 0, s>>>(g, nblk, w.blk_counts, map_out, w.ctl, offsets_out,
+                                                         g.phase == 2 ? g.nthr + 1 : 0));
 }
 
 // ---------------------------------------------------------------------------
@@ -373,8 +465,44 @@ __global__ void __launch_bounds__(1024) k_scan_final(const int* x, int n, const 
     }
 }
 
+// The three steps in one block for up to kScanSmall rows (one launch).
+constexpr int kScanSmall = 4 * kScanItems;
+
+__global__ void __launch_bounds__(1024) k_scan_small(const int* x, int n, Ctl* ctl, int* row_ptr) {
+    __shared__ long long scratch[33];
+    constexpr int kPer = kScanItems / 1024;
+    long long carry = 0;
+    for (int b0 = 0; b0 < n; b0 += kScanItems) {
+        const int base = b0 + (int)threadIdx.x * kPer;
+        int v[kPer];
+        long long sum = 0;
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            v[q] = base + q < n ? x[base + q] : 0;
+            sum += v[q];
+        }
+        long long tot;
+        long long ex = carry + block_excl_scan64(sum, scratch, &tot);
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            if (base + q < n) row_ptr[base + q] = (int)ex;
+            ex += v[q];
+        }
+        carry += tot;
+    }
+    if (threadIdx.x == 0) {
+        ctl->totals[2] = carry;
+        if (carry > 2147483647ll) set_status(ctl, ST_OVERFLOW);
+        row_ptr[n] = (int)carry;
+    }
+}
+
 void launch_row_ptr(const spgemm_plan* p, const int* row_nnz, int n, const WsPtrs& w,
                     int* row_ptr, cudaStream_t s) {
+    if (n <= kScanSmall) {
+        SPG_LAUNCH(p, K_SCAN_TOP, s, k_scan_small<<<1, 1024, 0, s>>>(row_nnz, n, w.ctl, row_ptr));
+        return;
+    }
     const int nscan = (n + kScanItems - 1) / kScanItems;
     if (nscan > 0)
         SPG_LAUNCH(p, K_SCAN_PART, s, k_scan_part<<<nscan, 1024, 0, s>>>(row_nnz, n, w.scan_part));

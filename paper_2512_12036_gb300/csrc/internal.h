@@ -160,6 +160,8 @@ struct WsLayout {
     size_t rc_bits = 0;      // u32 [rc_nslots][rc_wpr] row bitmaps of the allocation phase
     size_t rc_pc = 0;        // int [rc_nslots][panels] entries of each table panel of a cached row
     int rc_nslots = 0, rc_wpr = 0;
+    size_t nb_bits = 0;      // u32 [B.rows][nw] bitmaps of B's rows, nw = ceil(B.cols / 32)
+    size_t nc_bits = 0;      // u32 [m][nw]       and of C's rows (narrow tiers; B.cols <= kNarrowCols)
     bool has_hot = false;
     size_t total = 0;
     int m = 0, nblk = 0, nscan = 0, panels = 0;
@@ -184,6 +186,8 @@ struct WsPtrs {
     unsigned* rc_bits;
     int* rc_pc;              // per-panel entry counts of the cached rows, or nullptr
     int rc_nslots, rc_wpr;
+    unsigned* nb_bits;       // narrow tiers' bitmaps, or nullptr
+    unsigned* nc_bits;
     int nblk, nscan, panels, panel_cols;
 };
 
@@ -194,7 +198,6 @@ constexpr int kRowCacheMaxWords = 48 * 1024;   // one bitmap pass of the allocat
 WsPtrs ws_ptrs(const WsLayout& L, void* ws, int panel_cols);
 
 // Launchers (stream-ordered, no host synchronisation).
-void launch_fill_i64(const spgemm_plan* pl, long long* p, long long n, long long v, cudaStream_t s);
 void launch_ip_count(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, long long* ip,
                      const WsPtrs& w, cudaStream_t s);
 
@@ -222,13 +225,30 @@ void launch_row_ptr(const spgemm_plan* p, const int* row_nnz, int n, const WsPtr
 
 void launch_symbolic(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const long long* ip,
                      const WsPtrs& w, int* row_nnz, cudaStream_t s);
+void launch_check_rpt(const spgemm_plan* p, const CsrDev& M, const WsPtrs& w, cudaStream_t s);
 void launch_nnz_total(const spgemm_plan* p, const int* row_nnz, int n, const WsPtrs& w, cudaStream_t s);
 
+// Groups rows [row_begin, row_end) for the accumulation phase.
+void launch_numeric_group(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const long long* ip,
+                          int row_begin, int row_end, const int* rptC, const WsPtrs& w, cudaStream_t s);
+// The accumulation tiers of the grouped rows. bins: the grouping's bin starts
+// as the host has read them, or nullptr; with them only the tiers that have
+// rows are launched, and the dense tiers' tables of B are built here if one
+// of those has rows (without them the allocation phase has built them).
 // capacity >= 0: the tiers run only if rptC[n] <= capacity and no overflow
 // was flagged (otherwise ST_BUDGET is recorded and nothing is written).
+void launch_numeric_tiers(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, int row_begin,
+                          int row_end, const int* rptC, const WsPtrs& w, int* colC, float* valC,
+                          const int* bins, cudaStream_t s, long long capacity = -1);
+// Both.
 void launch_numeric(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const long long* ip,
                     int row_begin, int row_end, const int* rptC, const WsPtrs& w, int* colC,
                     float* valC, cudaStream_t s, long long capacity = -1);
+// Narrow tiers (narrow.cu).
+void launch_sym_narrow(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const WsPtrs& w,
+                       int* row_nnz, cudaStream_t s);
+void launch_num_narrow(const spgemm_plan* p, bool f64, const CsrDev& A, const CsrDev& B, const WsPtrs& w,
+                       const int* rptC, int row_begin, int* colC, float* valC, cudaStream_t s);
 // Bitmap tiers (bits.cu).
 bool bits_tier(const spgemm_plan* p, const CsrDev& B);
 int bits_cap(const spgemm_plan* p, const CsrDev& B, size_t acc);
@@ -237,6 +257,9 @@ void launch_sym_bits(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, con
 void launch_num_bits(const spgemm_plan* p, bool f64, const CsrDev& A, const CsrDev& B, const WsPtrs& w,
                      const int* rptC, int row_begin, int* colC, float* valC, int bin_lo, int bin_hi,
                      int tier, int cap, cudaStream_t s);
+// The tables of B that the dense accumulation tiers read (rows of more than
+// block_max_nnz entries; nothing where B has no more columns than that).
+void launch_dense_tables(const spgemm_plan* p, const CsrDev& B, const WsPtrs& w, cudaStream_t s);
 void launch_bpanel(const spgemm_plan* p, const CsrDev& B, const WsPtrs& w, cudaStream_t s);
 void launch_hot(const spgemm_plan* p, const CsrDev& B, const WsPtrs& w, cudaStream_t s);
 void launch_copy_total(const spgemm_plan* p, const WsPtrs& w, int which, long long* dst,

@@ -437,67 +437,6 @@ __global__ void __launch_bounds__(kSortWarps * 32) k_num_sort(CsrDev A, CsrDev B
     }
 }
 
-// Narrow B (<= kNarrowCols columns): one warp per row accumulates into a
-// per-warp dense array over all of B's columns (fp32, or fp64 for rows
-// where more than fp32_max_terms products can meet) and marks the columns in
-// a 32-word bitmap; lane l owns word l, so a warp scan of the popcounts
-// writes the row in column order with no sort. Touched entries are cleared
-// on the way out, so the array stays zero between rows.
-template <typename Acc>
-__global__ void __launch_bounds__(kNarrowMaxWarps * 32) k_num_narrow(CsrDev A, CsrDev B,
-                                                                     const int* map, Ctl* ctl,
-                                                                     const int* rptC, int row_begin,
-                                                                     int* colC, float* valC,
-                                                                     int bin, int ncols_pad) {
-    // per warp: a dense accumulator over B's columns, then a 32-word bitmap
-    extern __shared__ __align__(16) unsigned char sm_raw[];
-    const int warp = threadIdx.x >> 5, lane = lane_id();
-    const int nwarps = blockDim.x >> 5;
-    Acc* dense = reinterpret_cast<Acc*>(sm_raw) + warp * ncols_pad;
-    unsigned* bm = reinterpret_cast<unsigned*>(reinterpret_cast<Acc*>(sm_raw) + nwarps * ncols_pad) +
-                   warp * 32;
-    for (int c = lane; c < ncols_pad; c += 32) dense[c] = Acc(0);
-    bm[lane] = 0u;
-    __syncwarp();
-    const int begin = ctl->bin_off[bin], end = ctl->bin_off[bin + 1];
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int idx = begin + gw; idx < end; idx += nw) {
-        const int r = map[idx];
-        const int row = row_begin + r;
-        const int out = rptC[r];
-        const int nnz_row = rptC[r + 1] - out;
-        int rs, re;
-        row_extent(A, row, rs, re, ctl);
-        warp_expand(A, B, rs, re, 32, ctl, [&](int t, int ja) {
-            const int key = B.col[t];
-            if (key_in(key, B, ctl)) {
-                atomicOr(&bm[key >> 5], 1u << (key & 31));
-                atomicAdd(&dense[key], (Acc)A.val[ja] * (Acc)B.val[t]);
-            }
-        });
-        __syncwarp();
-        unsigned bits = bm[lane];
-        const int cnt = __popc(bits);
-        const int incl = warp_incl_scan(cnt);
-        int pos = incl - cnt;
-        const int tot = __shfl_sync(kFull, incl, 31);
-        while (bits) {
-            const int c = lane * 32 + __ffs(bits) - 1;
-            bits &= bits - 1;
-            if (pos < nnz_row) {
-                colC[out + pos] = c;
-                valC[out + pos] = (float)dense[c];
-            }
-            dense[c] = Acc(0);
-            ++pos;
-        }
-        bm[lane] = 0u;
-        if (lane == 0 && tot != nnz_row) set_status(ctl, ST_INTERNAL);
-        __syncwarp();
-    }
-}
-
 // ---------------------------------------------------------------------------
 // kT threads per block: kNumBlockThreads, or kBlockThreadsFull for the
 // launch whose full-size table leaves one block per SM (more warps to hide
@@ -1939,8 +1878,6 @@ void occupancy_numeric(spgemm_plan* p) {
         num_warp_kernel<double, 8>(wide, [&](const void* f, auto) { warp_occ(f, 8, 0, wide); });
         num_warp_kernel<double, 16>(wide, [&](const void* f, auto) { warp_occ(f, 8, 1, wide); });
     }
-    allow_max_dynamic_smem((const void*)k_num_narrow<float>, p);
-    allow_max_dynamic_smem((const void*)k_num_narrow<double>, p);
     for (auto& k : ks) {
         allow_max_dynamic_smem(k.f, p);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(k.occ, k.f, k.threads, k.smem);
@@ -1998,14 +1935,26 @@ static int dense_splits(const spgemm_plan* p, int panels) {
     return sp;
 }
 
+// Rows of the fp32 dense tier that the bitmap tier takes: up to this many
+// entries (0: none). Rows with cached bitmaps stay in the dense tiers, which
+// read them.
+static int num_bits_cap(const spgemm_plan* p, const CsrDev& B, const WsPtrs& w) {
+    return bits_tier(p, B) && !w.rc_slot ? bits_cap(p, B, sizeof(float)) : 0;
+}
+
 // Warp and block hash tiers: rows that outgrow the sort tier, for a B too
-// wide (or too narrow) for the bitmap tier.
+// wide (or too narrow) for the bitmap tier. below: every row of these tiers
+// has more products than that.
 static void launch_num_hash(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const int* rptC,
-                            int row_begin, const WsPtrs& w, int* colC, float* valC, cudaStream_t s) {
+                            int row_begin, const WsPtrs& w, int* colC, float* valC, const int* bins,
+                            long long below, cudaStream_t s) {
     const int sms = p->num_sms;
+    const spgemm_opts& o = p->opts;
+    auto has = [&](int bin) { return bins == nullptr || bins[bin + 1] > bins[bin]; };
     const bool wide = B.cols > kWarpPackCols;
     auto warp_tier = [&](int kid, size_t acc, int cls, int bin) {
         return [=](const void*, auto kernel) {
+            if (!has(bin) || 16ll * o.warp_max_nnz <= below) return;
             const int kN = kWarpClasses[cls];
             SPG_LAUNCH(p, kid, s,
                        kernel<<<sms * p->occ_num_warp[acc == 8][cls][wide], num_warp_warps(kN) * 32,
@@ -2021,40 +1970,34 @@ static void launch_num_hash(const spgemm_plan* p, const CsrDev& A, const CsrDev&
     // block hash tier: rows of more than half of block_max_nnz entries with
     // the full table (one block per SM), the others with a half- or
     // quarter-size table and as many blocks per SM as it leaves room for
-    const int max_bits = table_max_bits(num_block_smem(p, 4) / 8);
-    const int mid_bits = table_max_bits(num_block_smem_mid(p, 4) / 8);
-    const int small_bits = table_max_bits(num_block_smem_small(p, 4) / 8);
-    SPG_LAUNCH(p, K_NUM_BLOCK32, s,
-               k_num_block<float, kBlockThreadsFull><<<sms * p->occ_num_block32, kBlockThreadsFull,
-                                                      num_block_smem(p, 4), s>>>(
-                   A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_BLOCK32, 2, max_bits,
-                   hash_load(p)));
-    SPG_LAUNCH(p, K_NUM_BLOCK32, s,
-               k_num_block<float><<<sms * p->occ_num_block32m, kNumBlockThreads, num_block_smem_mid(p, 4), s>>>(
-                   A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_BLOCK32M, 10, mid_bits,
-                   hash_load(p)));
-    SPG_LAUNCH(p, K_NUM_BLOCK32, s,
-               k_num_block<float><<<sms * p->occ_num_block32s, kNumBlockThreads, num_block_smem_small(p, 4), s>>>(
-                   A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_BLOCK32S, 8, small_bits,
-                   hash_load(p)));
-    SPG_LAUNCH(p, K_NUM_BLOCK64, s,
-               k_num_block<double, kBlockThreadsFull><<<sms * p->occ_num_block64, kBlockThreadsFull,
-                                                       num_block_smem(p, 8), s>>>(
-                   A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_BLOCK64, 3, max_bits,
-                   hash_load(p)));
-    SPG_LAUNCH(p, K_NUM_BLOCK64, s,
-               k_num_block<double><<<sms * p->occ_num_block64m, kNumBlockThreads, num_block_smem_mid(p, 8), s>>>(
-                   A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_BLOCK64M, 11, mid_bits,
-                   hash_load(p)));
-    SPG_LAUNCH(p, K_NUM_BLOCK64, s,
-               k_num_block<double><<<sms * p->occ_num_block64s, kNumBlockThreads, num_block_smem_small(p, 8), s>>>(
-                   A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_BLOCK64S, 9, small_bits,
-                   hash_load(p)));
+    auto block_tier = [&](int kid, auto kernel, int occ, int threads, size_t smem, int bin, int tier, int above) {
+        if (has(bin) && B.cols > above)
+            SPG_LAUNCH(p, kid, s, kernel<<<sms * occ, threads, smem, s>>>(
+                A, B, w.map, w.ctl, rptC, row_begin, colC, valC, bin, tier,
+                table_max_bits(smem / (kid == K_NUM_BLOCK64 ? 12 : 8)), hash_load(p)));
+    };
+    block_tier(K_NUM_BLOCK32, k_num_block<float, kBlockThreadsFull>, p->occ_num_block32, kBlockThreadsFull,
+               num_block_smem(p, 4), NB_BLOCK32, 2, block_mid_nnz(o));
+    block_tier(K_NUM_BLOCK32, k_num_block<float>, p->occ_num_block32m, kNumBlockThreads,
+               num_block_smem_mid(p, 4), NB_BLOCK32M, 10, block_small_nnz(o));
+    block_tier(K_NUM_BLOCK32, k_num_block<float>, p->occ_num_block32s, kNumBlockThreads,
+               num_block_smem_small(p, 4), NB_BLOCK32S, 8, 0);
+    block_tier(K_NUM_BLOCK64, k_num_block<double, kBlockThreadsFull>, p->occ_num_block64, kBlockThreadsFull,
+               num_block_smem(p, 8), NB_BLOCK64, 3, block_mid_nnz(o));
+    block_tier(K_NUM_BLOCK64, k_num_block<double>, p->occ_num_block64m, kNumBlockThreads,
+               num_block_smem_mid(p, 8), NB_BLOCK64M, 11, block_small_nnz(o));
+    block_tier(K_NUM_BLOCK64, k_num_block<double>, p->occ_num_block64s, kNumBlockThreads,
+               num_block_smem_small(p, 8), NB_BLOCK64S, 9, 0);
 }
 
-void launch_numeric(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const long long* ip,
-                    int row_begin, int row_end, const int* rptC, const WsPtrs& w, int* colC,
-                    float* valC, cudaStream_t s, long long capacity) {
+void launch_dense_tables(const spgemm_plan* p, const CsrDev& B, const WsPtrs& w, cudaStream_t s) {
+    if (B.cols <= p->opts.block_max_nnz) return;
+    launch_bpanel(p, B, w, s);
+    launch_hot(p, B, w, s);
+}
+
+void launch_numeric_group(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const long long* ip,
+                          int row_begin, int row_end, const int* rptC, const WsPtrs& w, cudaStream_t s) {
     GroupArgs g{};
     g.phase = 1;
     g.row_begin = row_begin;
@@ -2064,30 +2007,44 @@ void launch_numeric(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, cons
     g.rptC = rptC;
     g.bcols = B.cols;
     g.rc_slot = w.rc_slot;
-    // rows with cached bitmaps stay in the dense tiers, which read them
-    g.bits_cap = bits_tier(p, B) && !w.rc_slot ? bits_cap(p, B, sizeof(float)) : 0;
+    g.bits_cap = num_bits_cap(p, B, w);
     g.opts = p->opts;
     launch_group(p, g, w, w.map, nullptr, s);
-    if (g.n == 0) return;
+}
+
+void launch_numeric(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const long long* ip,
+                    int row_begin, int row_end, const int* rptC, const WsPtrs& w, int* colC,
+                    float* valC, cudaStream_t s, long long capacity) {
+    launch_numeric_group(p, A, B, ip, row_begin, row_end, rptC, w, s);
+    launch_numeric_tiers(p, A, B, row_begin, row_end, rptC, w, colC, valC, nullptr, s, capacity);
+}
+
+void launch_numeric_tiers(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, int row_begin,
+                          int row_end, const int* rptC, const WsPtrs& w, int* colC, float* valC,
+                          const int* bins, cudaStream_t s, long long capacity) {
+    if (row_end == row_begin) return;
     if (capacity >= 0)
-        SPG_LAUNCH(p, K_GUARD, s, k_cap_guard<<<1, 64, 0, s>>>(rptC, g.n, capacity, w.ctl));
+        SPG_LAUNCH(p, K_GUARD, s, k_cap_guard<<<1, 64, 0, s>>>(rptC, row_end - row_begin, capacity, w.ctl));
     const int sms = p->num_sms;
-    SPG_LAUNCH(p, K_NUM_ESC, s, k_num_esc<<<sms * 8, 256, 0, s>>>(A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_ESC));
+    const spgemm_opts& o = p->opts;
+    // whether a row can be in bins [lo, hi): as read, else by the rules of the
+    // grouping that B's width decides (a narrow B leaves the hash and sort
+    // tiers only the rows beyond narrow_max_ip, and no row has more entries
+    // than B columns)
+    auto has = [&](int lo, int hi) { return bins == nullptr || bins[hi] > bins[lo]; };
+    const long long below = B.cols <= kNarrowCols ? narrow_max_ip(o) : 0;   // IP of any row past ESC and narrow
+    const int cap32 = num_bits_cap(p, B, w);
+    if (has(NB_ESC, NB_ESC + 1))
+        SPG_LAUNCH(p, K_NUM_ESC, s, k_num_esc<<<sms * 8, 256, 0, s>>>(A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_ESC));
     if (B.cols <= kNarrowCols) {
-        const int pad = (B.cols + 31) & ~31;
-        const int nwp = narrow_warps(p);
-        const int grid = sms * (64 / nwp > 1 ? 64 / nwp : 1);
-        SPG_LAUNCH(p, K_NUM_NARROW, s,
-                   k_num_narrow<float><<<grid, nwp * 32, (size_t)nwp * (pad * 4 + 128), s>>>(
-                       A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_NARROW32, pad));
-        SPG_LAUNCH(p, K_NUM_NARROW, s,
-                   k_num_narrow<double><<<grid, nwp * 32, (size_t)nwp * (pad * 8 + 128), s>>>(
-                       A, B, w.map, w.ctl, rptC, row_begin, colC, valC, NB_NARROW64, pad));
+        if (has(NB_NARROW32, NB_NARROW32 + 1)) launch_num_narrow(p, false, A, B, w, rptC, row_begin, colC, valC, s);
+        if (has(NB_NARROW64, NB_NARROW64 + 1)) launch_num_narrow(p, true, A, B, w, rptC, row_begin, colC, valC, s);
     }
-    if (B.cols < kSortCols) {
+    if (B.cols < kSortCols && sort_max_ip(o.warp_max_nnz) > below) {
         auto sort_tier = [&](int kid, auto kernel, int occ, int bin) {
-            SPG_LAUNCH(p, kid, s, kernel<<<sms * occ, kSortWarps * 32, 0, s>>>(
-                A, B, w.map, w.ctl, rptC, row_begin, colC, valC, bin));
+            if (has(bin, bin + 1))
+                SPG_LAUNCH(p, kid, s, kernel<<<sms * occ, kSortWarps * 32, 0, s>>>(
+                    A, B, w.map, w.ctl, rptC, row_begin, colC, valC, bin));
         };
         sort_tier(K_NUM_WARP32, k_num_sort<float, 16>, p->occ_num_sort[0][1], NB_SORT32B);
         sort_tier(K_NUM_WARP32, k_num_sort<float, 8>, p->occ_num_sort[0][0], NB_SORT32A);
@@ -2097,19 +2054,22 @@ void launch_numeric(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, cons
     if (bits_tier(p, B)) {
         // three sizes of row, so that the smaller ones leave room for more
         // blocks: up to twice warp_max_nnz, half of block_max_nnz and all
-        const spgemm_opts& o = p->opts;
         auto bits = [&](bool f64, int lo, int hi, int tier, int cap) {
-            launch_num_bits(p, f64, A, B, w, rptC, row_begin, colC, valC, lo, hi, tier, (cap + 3) & ~3, s);
+            if (has(lo, hi))
+                launch_num_bits(p, f64, A, B, w, rptC, row_begin, colC, valC, lo, hi, tier, (cap + 3) & ~3, s);
         };
-        if (g.bits_cap > 0) bits(false, NB_BITS32, NB_BITS32 + 1, 12, g.bits_cap);
+        if (cap32 > 0 && B.cols > o.block_max_nnz) bits(false, NB_BITS32, NB_BITS32 + 1, 12, cap32);
         bits(false, NB_BLOCK32, NB_BLOCK32 + 1, 2, o.block_max_nnz);
         bits(true, NB_BLOCK64, NB_BLOCK64 + 1, 3, o.block_max_nnz);
         bits(true, NB_WARP64S, NB_BLOCK64M + 1, 11, block_mid_nnz(o) > o.warp_max_nnz ? block_mid_nnz(o) : o.warp_max_nnz);
         bits(false, NB_BLOCK32S, NB_BLOCK32M + 1, 10, block_mid_nnz(o));
         bits(false, NB_WARP32S, NB_WARP32L + 1, 8, 2 * o.warp_max_nnz);
     } else {
-        launch_num_hash(p, A, B, rptC, row_begin, w, colC, valC, s);
+        launch_num_hash(p, A, B, rptC, row_begin, w, colC, valC, bins, below, s);
     }
+    // dense tiers: rows of more than block_max_nnz entries
+    if (B.cols <= o.block_max_nnz || !has(NB_DENSE32_0, NB_DENSE64_0 + NB_DENSE_N)) return;
+    if (bins) launch_dense_tables(p, B, w, s);
     const int PW = w.panel_cols;
     if (w.bhv && w.bpanel && B.nnz > 0)
         SPG_LAUNCH(p, K_HOT, s, k_pack_b<<<sms * 8, 256, 0, s>>>(B, w.bhot, w.bhv, w.bcv));

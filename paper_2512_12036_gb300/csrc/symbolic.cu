@@ -421,36 +421,6 @@ __global__ void k_rc_reset(int* rc_slot, int m, Ctl* ctl) {
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->rc_used = 0;
 }
 
-// Narrow B (<= kNarrowCols columns): one warp per row marks the row's
-// columns in a per-warp bitmap of 32 words (word w holds columns 32w..32w+31)
-// and counts them; no table, no probing.
-__global__ void __launch_bounds__(kNarrowMaxWarps * 32) k_sym_narrow(CsrDev A, CsrDev B,
-                                                                     const int* map, Ctl* ctl,
-                                                                     int* row_nnz, int bin) {
-    extern __shared__ unsigned bmw[];           // 32 words per warp
-    const int lane = lane_id();
-    unsigned* bm = bmw + (threadIdx.x >> 5) * 32;
-    bm[lane] = 0u;
-    __syncwarp();
-    const int begin = ctl->bin_off[bin], end = ctl->bin_off[bin + 1];
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int idx = begin + gw; idx < end; idx += nw) {
-        const int row = map[idx];
-        int rs, re;
-        row_extent(A, row, rs, re, ctl);
-        warp_expand(A, B, rs, re, 32, ctl, [&](int t, int) {
-            const int key = B.col[t];
-            if (key_ok(key, B, ctl)) atomicOr(&bm[key >> 5], 1u << (key & 31));
-        });
-        __syncwarp();
-        const int cnt = warp_sum(__popc(bm[lane]));
-        bm[lane] = 0u;
-        __syncwarp();
-        if (lane == 0) row_nnz[row] = cnt;
-    }
-}
-
 // ---------------------------------------------------------------------------
 
 // table of the block tier's two lighter bins: their rows hold at most
@@ -587,20 +557,23 @@ void launch_symbolic(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, con
     if (w.rc_slot)
         SPG_LAUNCH(p, K_FILL, s, k_rc_reset<<<sms * 4, 256, 0, s>>>(w.rc_slot, A.rows, w.ctl));
     SPG_LAUNCH(p, K_SYM_ESC, s, k_sym_esc<<<sms * 8, 256, 0, s>>>(A, B, w.map, w.ctl, row_nnz, SB_ESC));
-    SPG_LAUNCH(p, K_SYM_WARP, s,
-               k_sym_sort<16><<<sms * p->occ_sym_sort[1], kSortWarps * 32, 0, s>>>(
-                   A, B, w.map, w.ctl, row_nnz, SB_SORTB));
-    SPG_LAUNCH(p, K_SYM_WARP, s,
-               k_sym_sort<8><<<sms * p->occ_sym_sort[0], kSortWarps * 32, 0, s>>>(
-                   A, B, w.map, w.ctl, row_nnz, SB_SORTA));
+    // a narrow B leaves the other tiers only the rows beyond narrow_max_ip
+    const long long below = B.cols <= kNarrowCols ? narrow_max_ip(p->opts) : 0;
+    if (sort_max_ip(p->opts.warp_max_ip / 2) > below) {
+        SPG_LAUNCH(p, K_SYM_WARP, s,
+                   k_sym_sort<16><<<sms * p->occ_sym_sort[1], kSortWarps * 32, 0, s>>>(
+                       A, B, w.map, w.ctl, row_nnz, SB_SORTB));
+        SPG_LAUNCH(p, K_SYM_WARP, s,
+                   k_sym_sort<8><<<sms * p->occ_sym_sort[0], kSortWarps * 32, 0, s>>>(
+                       A, B, w.map, w.ctl, row_nnz, SB_SORTA));
+    }
     if (bits_tier(p, B)) launch_sym_bits(p, A, B, w, row_nnz, SB_WARP, SB_BLOCK0 + SB_BLOCK_N, 0, s);
-    else launch_sym_hash(p, A, B, ip, w, row_nnz, s);
-    if (B.cols <= kNarrowCols)
-        SPG_LAUNCH(p, K_SYM_NARROW, s,
-                   k_sym_narrow<<<sms * (64 / narrow_warps(p) > 1 ? 64 / narrow_warps(p) : 1),
-                                  narrow_warps(p) * 32, (size_t)narrow_warps(p) * 128, s>>>(
-                       A, B, w.map, w.ctl, row_nnz, SB_NARROW));
-    const size_t sd = sym_dense_smem(p);
+    else if (p->opts.block_max_ip > below) launch_sym_hash(p, A, B, ip, w, row_nnz, s);
+    if (B.cols <= kNarrowCols) launch_sym_narrow(p, A, B, w, row_nnz, s);
+    // no more of it than B's columns need: the rest of the SM's memory is L1
+    size_t sd = sym_dense_smem(p);
+    const size_t need = ((size_t)B.cols + 127) / 128 * 16;
+    if (need < sd) sd = need > 16 ? need : 16;
     SPG_LAUNCH(p, K_SYM_DENSE, s,
                k_sym_dense<<<sms * p->occ_sym_dense, kSymDenseThreads, sd, s>>>(
                    A, B, w.map, w.ctl, row_nnz, SB_DENSE0, SB_DENSE0 + SB_DENSE_N, 1, (int)(sd / 4),

@@ -1,0 +1,49 @@
+"""Narrow tiers (B of at most 1,024 columns): bitmap words and lane groups at
+their edges, B rows shorter and longer than a warp, repeated and unsorted
+columns, B's bitmaps built or not (A of many or few entries), fp32 and fp64
+rows, row blocks, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2512_12036_gb300 import DeviceCSR, Plan, gen
+from parity import compare
+
+pytestmark = pytest.mark.gpu
+
+
+def narrow_b(rows, cols, repeats, rng):
+    lens = rng.choice([0, 1, 2, 7, 31, 32, 33, 64, 65, 200], size=rows)
+    lens = np.minimum(lens, cols)
+    r = np.repeat(np.arange(rows), lens)
+    c = np.concatenate([rng.choice(cols, size=n, replace=False) for n in lens])
+    if repeats:
+        r, c = np.concatenate([r, r[::5]]), np.concatenate([c, c[::5]])
+        p = np.lexsort((rng.random(r.size), r))
+        r, c = r[p], c[p]
+    return gen.csr_from_coo(rows, cols, r, c, gen.uniform_open_closed(rng, r.size), sort=not repeats)
+
+
+@pytest.mark.parametrize("cols", [1, 31, 32, 33, 64, 100, 256, 257, 513, 1000, 1024])
+@pytest.mark.parametrize("repeats", [False, True])
+@pytest.mark.parametrize("few", [False, True])
+def test_narrow_rows(cols, repeats, few):
+    rng = np.random.default_rng(cols * 4 + 2 * repeats + few)
+    B = narrow_b(4000 if few else 700, cols, repeats, rng)
+    lens = rng.choice([0, 1, 3, 31, 32, 33, 40], size=40 if few else 300)
+    lens[:4] = 166, 168, 200, 300
+    r = np.repeat(np.arange(lens.size), lens)
+    c = rng.integers(0, B.rows, size=r.size)
+    A = gen.csr_from_coo(lens.size, B.rows, r, c, gen.uniform_open_closed(rng, r.size), sort=False)
+    assert (A.nnz >= B.rows // 2) == (not few)
+    ref = oracle.spgemm(A, B)
+    dA, dB = DeviceCSR.from_host(A), DeviceCSR.from_host(B)
+    for opts in ({}, {"narrow_warps": 16, "narrow_max_ip": 600}):
+        plan = Plan(**opts)
+        compare(plan.spgemm(dA, dB).to_host(), ref)
+        blocks, ip, nnz = plan.spgemm_blocks(dA, dB, max_block_nnz=max(1, int(ref.row_ptr[-1]) // 3 + 1024))
+        torch.cuda.synchronize()
+        assert nnz == int(ref.row_ptr[-1])
+        cols_out = np.concatenate([C.to_host().col for _, _, C in blocks])
+        assert np.array_equal(cols_out, ref.col)
