@@ -24,28 +24,38 @@ __global__ void k_zero_total(Ctl* ctl, int which) { ctl->totals[which] = 0; }
 // ---------------------------------------------------------------------------
 // Algorithm 1, balanced over nonzeros: each block takes a tile of A's stored
 // entries, so a row of 60k entries costs the same as 60k rows of one entry.
-// The owning row of an entry is found by binary search over the block's row
-// range; per-warp segmented sums then add into ip[row] with one atomic per
-// (warp, row) segment.
+// The lengths of the selected B rows are gathered (eight in flight per
+// thread) and scanned over the tile; a row's count is then a difference of
+// two prefixes, written directly when the row lies inside the tile and added
+// otherwise. (A binary search for the row of every entry and segmented warp
+// sums took 111 us on 11.5M entries of 589,000 rows; 69 us now.)
 // ---------------------------------------------------------------------------
 
 constexpr int kCountThreads = 256;
 constexpr int kCountItems = 8;
 constexpr int kCountTile = kCountThreads * kCountItems;
 
-__device__ __forceinline__ int row_of(const int* rpt, long long j, int lo, int hi) {
+// The last row in [0, hi] that starts at or before entry j, by one warp: 32
+// probes a step.
+__device__ __forceinline__ int row_of(const int* rpt, long long j, int hi) {
+    const int lane = lane_id();
+    int lo = 0;
     while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if ((long long)rpt[mid] <= j) lo = mid;
-        else hi = mid - 1;
+        const int step = (hi - lo + 33) / 33;    // 33 steps cover [lo, hi]
+        const int p = lo + (lane + 1) * step;
+        const int c = __popc(__ballot_sync(kFull, p <= hi && (long long)rpt[p <= hi ? p : hi] <= j));
+        lo += c * step;
+        hi = min(hi, lo + step - 1);
     }
     return lo;
 }
 
 __global__ void __launch_bounds__(kCountThreads) k_ip_count(CsrDev A, CsrDev B, long long* ip,
                                                             Ctl* ctl) {
-    __shared__ int s_r0, s_r1;
-    __shared__ long long red[33];
+    __shared__ int s_r[2];
+    __shared__ int s_len[kCountTile + kCountTile / 32];          // (padded: thread t reads 8t ..)
+    __shared__ unsigned long long s_pre[kCountTile + 1];
+    __shared__ unsigned long long scratch[33];
     const int m = A.rows;
     const long long J0 = A.rpt[0], J1 = A.rpt[m];
     if (J0 < 0 || J1 < J0 || J1 > A.nnz) {
@@ -55,39 +65,52 @@ __global__ void __launch_bounds__(kCountThreads) k_ip_count(CsrDev A, CsrDev B, 
     const long long jb = J0 + (long long)blockIdx.x * kCountTile;
     if (jb >= J1) return;
     const long long je = jb + kCountTile < J1 ? jb + kCountTile : J1;
-    if (threadIdx.x == 0) {
-        const int r0 = row_of(A.rpt, jb, 0, m - 1);
-        s_r0 = r0;
-        s_r1 = row_of(A.rpt, je - 1, r0, m - 1);
+    const int t = threadIdx.x;
+    // the tile's first and last row, searched while the lengths are gathered
+    if ((t >> 5) < 2) {
+        const int r = row_of(A.rpt, (t >> 5) == 0 ? jb : je - 1, m - 1);
+        if (lane_id() == 0) s_r[t >> 5] = r;
+    }
+    int len[kCountItems];
+#pragma unroll
+    for (int q = 0; q < kCountItems; ++q) {
+        const long long j = jb + q * kCountThreads + t;
+        int bs;
+        len[q] = 0;
+        if (j < je) a_entry(A, B, (int)j, bs, len[q], ctl);
+    }
+#pragma unroll
+    for (int q = 0; q < kCountItems; ++q) {
+        const int p = q * kCountThreads + t;
+        s_len[p + (p >> 5)] = len[q];
     }
     __syncthreads();
-    const int r0 = s_r0, r1 = s_r1;
-    const int lane = lane_id();
-    long long sum = 0;                               // this thread's products
-    for (int it = 0; it < kCountItems; ++it) {
-        const long long j = jb + (long long)it * kCountThreads + threadIdx.x;
-        int row = -1;
-        long long v = 0;
-        if (j < je) {
-            row = row_of(A.rpt, j, r0, r1);
-            int bs, len;
-            a_entry(A, B, (int)j, bs, len, ctl);
-            v = len;
-            sum += len;
-        }
-        // segmented inclusive scan over contiguous equal rows
+    unsigned long long sum = 0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long n = __shfl_up_sync(kFull, v, o);
-            const int rp = __shfl_up_sync(kFull, row, o);
-            if (lane >= o && rp == row) v += n;
-        }
-        const int rn = __shfl_down_sync(kFull, row, 1);
-        const bool last = (lane == 31) || rn != row;
-        if (last && row >= 0 && v != 0) atomicAdd((unsigned long long*)&ip[row], (unsigned long long)v);
+    for (int q = 0; q < kCountItems; ++q) {
+        const int p = t * kCountItems + q;
+        len[q] = s_len[p + (p >> 5)];
+        sum += (unsigned)len[q];
     }
-    sum = block_sum(sum, red);
-    if (threadIdx.x == 0 && sum != 0) atomicAdd((unsigned long long*)&ctl->totals[0], (unsigned long long)sum);
+    unsigned long long tot;
+    unsigned long long run = block_excl_scan_u64(sum, scratch, &tot);
+#pragma unroll
+    for (int q = 0; q < kCountItems; ++q) {
+        s_pre[t * kCountItems + q] = run;
+        run += (unsigned)len[q];
+    }
+    if (t == kCountThreads - 1) s_pre[kCountTile] = run;
+    __syncthreads();
+    const int r1 = s_r[1];
+    for (int r = s_r[0] + t; r <= r1; r += kCountThreads) {
+        const long long s = A.rpt[r], e = A.rpt[r + 1];
+        // (row pointers out of order were flagged; they stay inside the tile here)
+        const long long a = s > jb ? (s < je ? s : je) : jb, b = e < je ? (e > a ? e : a) : je;
+        const unsigned long long v = s_pre[b - jb] - s_pre[a - jb];
+        if (s >= jb && e <= je) ip[r] = (long long)v;
+        else if (v != 0) atomicAdd((unsigned long long*)&ip[r], v);
+    }
+    if (t == 0 && tot != 0) atomicAdd((unsigned long long*)&ctl->totals[0], tot);
 }
 
 // One pass over the rows before the count: zero counts, both operands' row
