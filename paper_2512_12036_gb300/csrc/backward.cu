@@ -176,7 +176,7 @@ __device__ __forceinline__ float warp_sum4(const float (&v)[4]) {
 // all loads first, then the look-ups, the dB atomics and one joint reduction
 // for the four dA. What bounds it: the fp64 atomics into L2 and instruction
 // issue (589,000 rows of 612 products over 256 columns: 1,982 us with the
-// general chunk above, 1,251 us here).
+// general chunk above, 1,022 us here).
 __global__ void __launch_bounds__(kBwdWarps * 32, 5) k_bwd_dense(BwdArgs x, int bin) {
     extern __shared__ float sm_dense[];
     const int begin = x.ctl->bin_off[bin], end = x.ctl->bin_off[bin + 1];
@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 5) k_bwd_dense(BwdArgs x, int 
                 continue;
             }
             float mine = 0.f;
+            const bool one_step = !__any_sync(kFull, len > 32);      // a product per lane, no loops
             for (int q = 0; q < cnt; q += 4) {
                 int ts[4], tl[4], c[4];
                 float av[4], b[4], acc[4];
@@ -239,6 +240,19 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 5) k_bwd_dense(BwdArgs x, int 
                         b[u] = x.B.val[ts[u]];
                     }
                 }
+                if (one_step) {
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        acc[u] = 0.f;
+                        if ((unsigned)c[u] < (unsigned)cols) {
+                            const float g = dense[c[u]];
+                            acc[u] = g * b[u];
+                            if (x.dB64) atomicAdd(&x.dB64[ts[u]], bwd_widen(av[u] * g));
+                        } else if (lane < tl[u]) {
+                            set_status(x.ctl, ST_INVALID);
+                        }
+                    }
+                } else {
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     acc[u] = 0.f;
@@ -260,6 +274,7 @@ __global__ void __launch_bounds__(kBwdWarps * 32, 5) k_bwd_dense(BwdArgs x, int 
                             }
                         }
                     }
+                }
                 }
                 if (x.dA) {
                     const float sum = warp_sum4(acc);
