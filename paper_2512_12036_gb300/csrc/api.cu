@@ -11,7 +11,6 @@ void occupancy_numeric(spgemm_plan* p);
 void occupancy_bits(spgemm_plan* p);
 void occupancy_narrow(spgemm_plan* p);
 void occupancy_backward(spgemm_plan* p);
-void occupancy_mcl(spgemm_plan* p);
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 WsLayout ws_layout(const spgemm_plan* p, long long m, long long b_rows, long long b_cols,
@@ -32,6 +31,8 @@ WsLayout ws_layout(const spgemm_plan* p, long long m, long long b_rows, long lon
     off = align256(off + sizeof(int) * (size_t)kNumBins * (size_t)(L.nblk > 0 ? L.nblk : 1));
     L.scan_part = off;
     off = align256(off + sizeof(long long) * (size_t)(L.nscan + 1));
+    L.row_scratch = off;
+    off = align256(off + 3 * sizeof(int) * (size_t)(m > 0 ? m : 1));
     L.bpanel = off;
     if (L.panels > 0 && L.panels <= kMaxPanels && b_rows > 0)
         off = align256(off + sizeof(int) * (size_t)b_rows * (size_t)(L.panels + 1));
@@ -89,6 +90,7 @@ WsPtrs ws_ptrs(const WsLayout& L, void* ws, int panel_cols) {
     w.map = (int*)(b + L.map);
     w.blk_counts = (int*)(b + L.blk_counts);
     w.scan_part = (long long*)(b + L.scan_part);
+    w.row_scratch = (int*)(b + L.row_scratch);
     w.bpanel = (L.panels > 0 && L.panels <= kMaxPanels && (L.has_hot ? L.colcnt : L.total) > L.bpanel)
                    ? (int*)(b + L.bpanel) : nullptr;
     w.colcnt = L.has_hot ? (int*)(b + L.colcnt) : nullptr;
@@ -125,7 +127,6 @@ void init_occupancy(spgemm_plan* p) {
     occupancy_bits(p);
     occupancy_narrow(p);
     occupancy_backward(p);
-    occupancy_mcl(p);
 }
 
 const char* const kKernelNames[K_NUM_KERNELS] = {

@@ -149,6 +149,7 @@ struct WsLayout {
     size_t map = 0;          // int32 [m]
     size_t blk_counts = 0;   // int32 [kNumBins][nblk]
     size_t scan_part = 0;    // int64 [nscan + 1]
+    size_t row_scratch = 0;  // int32 [3][m]      (Markov-clustering step)
     size_t bpanel = 0;       // int32 [B.rows][P+1]  (0 bytes when P > kMaxPanels)
     size_t colcnt = 0;       // int32 [B.cols+1]  entries per column of B, then hot flags
     size_t hot_rank = 0;     // int32 [B.cols+1]  exclusive prefix of the hot flags
@@ -175,6 +176,7 @@ struct WsPtrs {
     int* map;
     int* blk_counts;
     long long* scan_part;
+    int* row_scratch;
     int* bpanel;
     int* colcnt;
     int* hot_rank;

@@ -8,7 +8,11 @@
 // inflate first). The k-th largest decision value is found by a radix
 // selection over order-preserving 32-bit keys (four 8-bit digits, a
 // 256-bin histogram each), so no sort is needed; kept entries keep their
-// column order.
+// column order. Selection runs once: it leaves the threshold key of every row
+// for the writing pass, which filters by it, stages the kept values in the
+// output and inflates and normalises only those. (With the selection run
+// again before writing, and pow inlined into unrolled loops beyond the
+// instruction cache, 50,021 rows of 600 entries took 3,343 us; 511 us now.)
 // Weights and the row sum are fp64; each output is rounded once to fp32.
 // k < 0 keeps every entry that passes the threshold (a plain normalisation
 // when theta <= 0 and r = 1).
@@ -16,11 +20,9 @@
 
 namespace spg {
 
-constexpr int kMclWarpMax = 1024;     // rows up to this length: one warp, 32 entries per lane
+constexpr int kMclWarpMax = 1024;     // rows up to this length: one warp, 32 keys per lane
 constexpr int kMclThreads = 256;
-constexpr int kMclBlockThreads = 1024;
-constexpr int kMclStage = 32768;      // decision keys of a block row kept in shared memory (128 KB)
-constexpr int kMclChunk = 128;        // rows the block kernel looks at together
+constexpr int kMclStage = 6144;       // decision keys of a longer row kept in shared memory
 
 struct MclParams {
     float theta;
@@ -29,29 +31,48 @@ struct MclParams {
     int order;
 };
 
+// Scratch of a step: per row the k-th largest decision key and how many
+// entries equal to it are kept, and the list of rows above kMclWarpMax.
+struct MclScratch {
+    unsigned* thr;
+    int* need;
+    int* longer;
+};
+
 __device__ __forceinline__ unsigned ord_key(float x) {
     const unsigned b = __float_as_uint(x);
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
 }
 
+// (out of line: inlined into unrolled loops, pow overran the instruction cache)
+__device__ __noinline__ double mcl_pow(double d, double r) { return pow(d, r); }
+
 __device__ __forceinline__ double mcl_weight(float v, double r) {
     const double d = (double)v;
     if (r == 2.0) return d * d;
     if (r == 1.0) return d;
-    return pow(d, r);
+    return mcl_pow(d, r);
 }
 
+// (the product of two fp32 numbers is exact in fp64, so rounding it to fp32
+// is the fp32 product)
 __device__ __forceinline__ float mcl_decide(float v, const MclParams& p) {
-    return p.order == 0 ? v : (float)mcl_weight(v, p.r);
+    if (p.order == 0 || p.r == 1.0) return v;
+    return p.r == 2.0 ? __fmul_rn(v, v) : (float)mcl_weight(v, p.r);
+}
+
+__device__ __forceinline__ unsigned mcl_key(float v, const MclParams& p) {
+    const float d = mcl_decide(v, p);
+    return d >= p.theta ? ord_key(d) : 0u;       // 0: pruned
 }
 
 // ---------------------------------------------------------------------------
-// One warp per row of length <= kMclWarpMax. kWrite = false: count the kept
-// entries into counts[row]; true: write them at rpt_out[row].
-template <bool kWrite>
-__global__ void __launch_bounds__(kMclThreads) k_mcl_warp(CsrDev E, MclParams prm, int* counts,
-                                                          const int* rpt_out, int* col_out,
-                                                          float* val_out, Ctl* ctl) {
+// Selection, rows of up to kMclWarpMax entries: one warp per row. The kept
+// entries are those above the k-th largest key and the first few equal to it;
+// key and number go to the scratch, their count to counts[row]. Longer rows
+// are listed for k_mcl_select_long.
+__global__ void __launch_bounds__(kMclThreads) k_mcl_select(CsrDev E, MclParams prm, int* counts,
+                                                            MclScratch ms, Ctl* ctl) {
     constexpr int kPer = kMclWarpMax / 32;
     __shared__ int whist[kMclThreads / 32][256];
     const int lane = lane_id();
@@ -62,37 +83,38 @@ __global__ void __launch_bounds__(kMclThreads) k_mcl_warp(CsrDev E, MclParams pr
         int s, e;
         row_extent(E, (int)row, s, e, ctl);
         const int n = e - s;
-        if (n > kMclWarpMax) continue;                       // block kernel's row
+        if (n > kMclWarpMax) {
+            if (lane == 0) ms.longer[atomicAdd(&ctl->work[0], 1)] = (int)row;
+            continue;
+        }
         unsigned key[kPer];
         int cnt = 0;
 #pragma unroll
         for (int i = 0; i < kPer; ++i) {
-            const int q = s + lane + 32 * i;
             key[i] = 0u;
-            if (q < e) {
-                const float d = mcl_decide(E.val[q], prm);
-                if (d >= prm.theta) {
-                    key[i] = ord_key(d);
-                    ++cnt;
-                }
+            if (32 * i < n) {                                   // warp-uniform
+                const int q = s + lane + 32 * i;
+                if (q < e) key[i] = mcl_key(E.val[q], prm);
+                cnt += key[i] != 0u;
             }
         }
-        cnt = warp_sum(cnt);
+        cnt = __reduce_add_sync(kFull, cnt);
         const bool cut = prm.k >= 0 && cnt > prm.k;
-        unsigned K = 1u;
-        int need_eq = 0;
+        unsigned K = 0u;
+        int need = 0;
         if (cut) {
             // the k-th largest key by radix selection, 8 bits a pass from the
-            // top, on a per-warp 256-bin histogram (see mcl_radix_digit)
+            // top, on a per-warp 256-bin histogram
             unsigned prefix = 0u, pmask = 0u;
             int above = 0;
+#pragma unroll 1
             for (int sh = 24; sh >= 0; sh -= 8) {
 #pragma unroll
-                for (int b = 0; b < 8; ++b) hist[8 * lane + b] = 0;
+                for (int b = 0; b < 8; ++b) hist[lane + 32 * b] = 0;
                 __syncwarp();
 #pragma unroll
                 for (int i = 0; i < kPer; ++i)
-                    if (key[i] != 0u && (key[i] & pmask) == prefix)
+                    if (32 * i < n && key[i] != 0u && (key[i] & pmask) == prefix)
                         atomicAdd(&hist[(key[i] >> sh) & 255u], 1);
                 __syncwarp();
                 int dig, run_at;
@@ -103,129 +125,51 @@ __global__ void __launch_bounds__(kMclThreads) k_mcl_warp(CsrDev E, MclParams pr
                 __syncwarp();
             }
             K = prefix;
-            need_eq = prm.k - above;
+            need = prm.k - above;
         }
-        const int keep_n = cut ? prm.k : cnt;
-        if (!kWrite) {
-            if (lane == 0) counts[row] = keep_n;
-            continue;
+        if (lane == 0) {
+            counts[row] = cut ? prm.k : cnt;
+            ms.thr[row] = K;                                    // (0: every unpruned entry)
+            ms.need[row] = need;
         }
-        // pass 1: kept flags in column order, weight sum
-        unsigned keepmask = 0u;
-        int eq_seen = 0;
-        double wsum = 0.0;
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            const bool cand = key[i] != 0u;
-            bool kp = cand;
-            if (cut) {                               // warp-uniform branch
-                const bool eq = cand && key[i] == K;
-                const unsigned eqb = __ballot_sync(kFull, eq);
-                const int rank = eq_seen + __popc(eqb & lanemask_lt());
-                kp = cand && (key[i] > K || (eq && rank < need_eq));
-                eq_seen += __popc(eqb);
-            }
-            if (kp) {
-                keepmask |= 1u << i;
-                wsum += mcl_weight(E.val[s + lane + 32 * i], prm.r);
-            }
-        }
-        wsum = warp_sum(wsum);
-        // pass 2: write in column order
-        int pos = rpt_out[row];
-        const int pend = rpt_out[row + 1];
-#pragma unroll
-        for (int i = 0; i < kPer; ++i) {
-            const bool kp = (keepmask >> i) & 1u;
-            const unsigned b = __ballot_sync(kFull, kp);
-            if (kp) {
-                const int q = s + lane + 32 * i;
-                const int o = pos + __popc(b & lanemask_lt());
-                if (o < pend) {
-                    col_out[o] = E.col[q];
-                    const double w = mcl_weight(E.val[q], prm.r);
-                    val_out[o] = wsum > 0.0 ? (float)(w / wsum) : 0.f;
-                } else {
-                    set_status(ctl, ST_INTERNAL);
-                }
-            }
-            pos += __popc(b);
-        }
-        if (lane == 0 && pos != pend) set_status(ctl, ST_INTERNAL);
     }
 }
 
-// ---------------------------------------------------------------------------
-// One block per row of length > kMclWarpMax (picked from chunks of rows). The
-// row's decision keys are computed once into shared memory (rows up to
-// kMclStage entries; longer rows recompute them per pass) and the k-th
-// largest is found by a 4-pass radix selection (8 bits a pass).
-template <bool kWrite>
-__global__ void __launch_bounds__(kMclBlockThreads) k_mcl_block(CsrDev E, MclParams prm,
-                                                                int* counts, const int* rpt_out,
-                                                                int* col_out, float* val_out,
-                                                                Ctl* ctl) {
+// The same for a listed row per block: its keys in shared memory (rows of up
+// to kMclStage entries; longer ones compute them again each pass).
+__global__ void __launch_bounds__(kMclThreads) k_mcl_select_long(CsrDev E, MclParams prm, int* counts,
+                                                                 MclScratch ms, Ctl* ctl) {
     __shared__ int red[33];
-    __shared__ double redd[33];
-    __shared__ int scratch[33];
     __shared__ int hist[256];
-    __shared__ int s_dig, s_above;
-    extern __shared__ unsigned skey[];             // kMclStage decision keys
-    __shared__ int s_long[kMclBlockThreads];       // this chunk's rows above kMclWarpMax
-    __shared__ int s_nlong;
-    // chunks of kMclChunk consecutive rows: one parallel look at their
-    // lengths picks this kernel's rows, which the block then takes one at a
-    // time (small chunks keep the blocks' shares of long rows even)
-    for (long long base = (long long)blockIdx.x * kMclChunk; base < E.rows;
-         base += (long long)gridDim.x * kMclChunk) {
-    {
-        const long long r0 = base + threadIdx.x;
-        bool is_long = false;
-        if ((int)threadIdx.x < kMclChunk && r0 < E.rows) {
-            const int rs0 = E.rpt[r0], re0 = E.rpt[r0 + 1];
-            is_long = re0 - rs0 > kMclWarpMax;
-        }
-        int nl;
-        const int slot = block_excl_scan(is_long ? 1 : 0, scratch, &nl);
-        if (is_long) s_long[slot] = (int)r0;
-        if (threadIdx.x == 0) s_nlong = nl;
+    __shared__ int s_li, s_dig, s_above;
+    __shared__ unsigned skey[kMclStage];
+    const int nlong = ctl->work[0];
+    for (;;) {
+        if (threadIdx.x == 0) s_li = atomicAdd(&ctl->work[1], 1);
         __syncthreads();
-    }
-    const int nlong = s_nlong;
-    for (int li = 0; li < nlong; ++li) {
-        const long long row = s_long[li];
+        const int li = s_li;
+        if (li >= nlong) break;
+        const int row = ms.longer[li];
         int s, e;
-        row_extent(E, (int)row, s, e, ctl);
-        if (e - s <= kMclWarpMax) continue;
-        auto key_of = [&](int q) -> unsigned {
-            const float d = mcl_decide(E.val[q], prm);
-            return d >= prm.theta ? ord_key(d) : 0u;
-        };
-        // decision keys, staged in shared memory when the row fits
+        row_extent(E, row, s, e, ctl);
         const int n = e - s;
         const bool staged = n <= kMclStage;
         int c0 = 0;
-        for (int q = s + threadIdx.x; q < e; q += blockDim.x) {
-            const unsigned kq = key_of(q);
-            if (staged) skey[q - s] = kq;
+        for (int q = threadIdx.x; q < n; q += kMclThreads) {
+            const unsigned kq = mcl_key(E.val[s + q], prm);
+            if (staged) skey[q] = kq;
             c0 += kq != 0u;
         }
-        const int cnt = block_sum(c0, red);       // (barrier: skey ready)
-        auto key_at = [&](int q) -> unsigned { return staged ? skey[q - s] : key_of(q); };
+        const int cnt = block_sum(c0, red);                     // (barrier: skey ready)
         const bool cut = prm.k >= 0 && cnt > prm.k;
-        unsigned K = 1u;
-        int need_eq = 0;
+        unsigned prefix = 0u, pmask = 0u;
+        int above = 0;
         if (cut) {
-            // the k-th largest key by radix selection, 8 bits a pass from the
-            // top: a 256-bin histogram of the keys that share the prefix found
-            // so far, then the digit whose bin holds the k-th largest
-            unsigned prefix = 0u, pmask = 0u;
-            int above = 0;                          // keys known to be larger than the prefix
             for (int sh = 24; sh >= 0; sh -= 8) {
-                for (int b = threadIdx.x; b < 256; b += blockDim.x) hist[b] = 0;
+                hist[threadIdx.x] = 0;
                 __syncthreads();
-                for (int q = s + threadIdx.x; q < e; q += blockDim.x) {
-                    const unsigned kq = key_at(q);
+                for (int q = threadIdx.x; q < n; q += kMclThreads) {
+                    const unsigned kq = staged ? skey[q] : mcl_key(E.val[s + q], prm);
                     if (kq != 0u && (kq & pmask) == prefix) atomicAdd(&hist[(kq >> sh) & 255u], 1);
                 }
                 __syncthreads();
@@ -241,67 +185,142 @@ __global__ void __launch_bounds__(kMclBlockThreads) k_mcl_block(CsrDev E, MclPar
                 prefix |= (unsigned)s_dig << sh;
                 pmask |= 255u << sh;
                 above = s_above;
-                __syncthreads();
             }
-            K = prefix;
-            need_eq = prm.k - above;
         }
-        const int keep_n = cut ? prm.k : cnt;
-        if (!kWrite) {
-            if (threadIdx.x == 0) counts[row] = keep_n;
-            continue;
+        if (threadIdx.x == 0) {
+            counts[row] = cut ? prm.k : cnt;
+            ms.thr[row] = prefix;
+            ms.need[row] = cut ? prm.k - above : 0;
         }
-        // chunks of blockDim entries in column order: kept flags, then writes
-        auto kept = [&](int q, unsigned kq, int eq_rank) {
-            if (kq == 0u) return false;
-            if (!cut) return true;
-            if (kq > K) return true;
-            return kq == K && eq_rank < need_eq;
-        };
-        double wpart = 0.0;
-        int eq_seen = 0;
-        for (int base = s; base < e; base += blockDim.x) {
-            const int q = base + threadIdx.x;
-            const unsigned kq = q < e ? key_of(q) : 0u;
-            int eq_tot;
-            const int eq_rank = eq_seen + block_excl_scan((cut && kq == K) ? 1 : 0, scratch, &eq_tot);
-            if (q < e && kept(q, kq, eq_rank)) wpart += mcl_weight(E.val[q], prm.r);
-            eq_seen += eq_tot;
-        }
-        const double wsum = block_sum(wpart, redd);
-        int pos = rpt_out[row];
-        const int pend = rpt_out[row + 1];
-        eq_seen = 0;
-        for (int base = s; base < e; base += blockDim.x) {
-            const int q = base + threadIdx.x;
-            const unsigned kq = q < e ? key_of(q) : 0u;
-            int eq_tot;
-            const int eq_rank = eq_seen + block_excl_scan((cut && kq == K) ? 1 : 0, scratch, &eq_tot);
-            eq_seen += eq_tot;
-            const bool kp = q < e && kept(q, kq, eq_rank);
-            int ktot;
-            const int o = pos + block_excl_scan(kp ? 1 : 0, scratch, &ktot);
-            if (kp) {
-                if (o < pend) {
-                    col_out[o] = E.col[q];
-                    const double w = mcl_weight(E.val[q], prm.r);
-                    val_out[o] = wsum > 0.0 ? (float)(w / wsum) : 0.f;
-                } else {
-                    set_status(ctl, ST_INTERNAL);
-                }
-            }
-            pos += ktot;
-        }
-        if (threadIdx.x == 0 && pos != pend) set_status(ctl, ST_INTERNAL);
         __syncthreads();
-    }
-    __syncthreads();                               // s_long is rewritten by the next chunk
     }
 }
 
-void occupancy_mcl(spgemm_plan* p) {
-    allow_max_dynamic_smem((const void*)k_mcl_block<false>, p);
-    allow_max_dynamic_smem((const void*)k_mcl_block<true>, p);
+// ---------------------------------------------------------------------------
+// Writing: a warp takes entries [q0, q1) of a row in column order, the kept
+// ones going to [pos, pend) as (column, value), `eq` of those equal to the
+// threshold key being already taken. Returns the position after the last.
+// Four groups of 32 are loaded at a time.
+__device__ __forceinline__ int mcl_write(const CsrDev& E, const MclParams& prm, unsigned K, int need,
+                                         bool cut, int q0, int q1, int pos, int pend, int& eq,
+                                         int* col_out, float* val_out) {
+    const int lane = lane_id();
+    for (int b = q0; b < q1; b += 128) {
+        float v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = b + 32 * u + lane < q1 ? E.val[b + 32 * u + lane] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int q = b + 32 * u + lane;
+            if (b + 32 * u >= q1) break;                        // warp-uniform
+            const unsigned key = q < q1 ? mcl_key(v[u], prm) : 0u;
+            bool keep = key > K;
+            if (cut) {
+                const unsigned eqb = __ballot_sync(kFull, key == K && key != 0u);
+                if (eqb) {
+                    keep |= key == K && key != 0u && eq + __popc(eqb & lanemask_lt()) < need;
+                    eq += __popc(eqb);
+                }
+            }
+            const unsigned kb = __ballot_sync(kFull, keep);
+            if (keep) {
+                const int o = pos + __popc(kb & lanemask_lt());
+                if (o < pend) {
+                    col_out[o] = E.col[q];
+                    val_out[o] = v[u];
+                }
+            }
+            pos += __popc(kb);
+        }
+    }
+    return pos;
+}
+
+// Inflate and normalise kept values in place: w / sum of w, fp64.
+template <int kT>
+__device__ __forceinline__ double mcl_weights(const float* val, int a, int b, int t, double r) {
+    double sum = 0.0;
+    for (int q = a + t; q < b; q += kT) sum += mcl_weight(val[q], r);
+    return sum;
+}
+
+__global__ void __launch_bounds__(kMclThreads) k_mcl_write(CsrDev E, MclParams prm, MclScratch ms,
+                                                           const int* rpt_out, int* col_out,
+                                                           float* val_out, Ctl* ctl) {
+    const int lane = lane_id();
+    const long long gw = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+    const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
+    for (long long row = gw; row < E.rows; row += nw) {
+        int s, e;
+        row_extent(E, (int)row, s, e, ctl);
+        if (e - s > kMclWarpMax) continue;
+        const unsigned K = ms.thr[row];
+        const int need = ms.need[row];
+        const int p0 = rpt_out[row], p1 = rpt_out[row + 1];
+        const bool cut = prm.k >= 0 && p1 - p0 == prm.k;
+        int eq = 0;
+        const int pos = mcl_write(E, prm, K, need, cut, s, e, p0, p1, eq, col_out, val_out);
+        if (lane == 0 && pos != p1) set_status(ctl, ST_INTERNAL);
+        __syncwarp();
+        const double sum = warp_sum(mcl_weights<32>(val_out, p0, p1, lane, prm.r));
+        for (int q = p0 + lane; q < p1; q += 32)
+            val_out[q] = sum > 0.0 ? (float)(mcl_weight(val_out[q], prm.r) / sum) : 0.f;
+    }
+}
+
+// A listed row per block, a contiguous share of it per warp: every warp
+// counts the entries above and at the threshold in its share first.
+__global__ void __launch_bounds__(kMclThreads) k_mcl_write_long(CsrDev E, MclParams prm, MclScratch ms,
+                                                                const int* rpt_out, int* col_out,
+                                                                float* val_out, Ctl* ctl) {
+    constexpr int kWarps = kMclThreads / 32;
+    __shared__ int s_li;
+    __shared__ int s_gt[kWarps], s_eq[kWarps];
+    __shared__ double redd[33];
+    const int lane = lane_id(), warp = threadIdx.x >> 5;
+    const int nlong = ctl->work[0];
+    for (;;) {
+        if (threadIdx.x == 0) s_li = atomicAdd(&ctl->work[2], 1);
+        __syncthreads();
+        const int li = s_li;
+        if (li >= nlong) break;
+        const int row = ms.longer[li];
+        int s, e;
+        row_extent(E, row, s, e, ctl);
+        const unsigned K = ms.thr[row];
+        const int need = ms.need[row];
+        const int p0 = rpt_out[row], p1 = rpt_out[row + 1];
+        const bool cut = prm.k >= 0 && p1 - p0 == prm.k;
+        const int per = ((e - s + kWarps - 1) / kWarps + 31) & ~31;
+        const int q0 = s + warp * per < e ? s + warp * per : e;
+        const int q1 = q0 + per < e ? q0 + per : e;
+        int gt = 0, at = 0;
+        for (int q = q0 + lane; q < q1; q += 32) {
+            const unsigned key = mcl_key(E.val[q], prm);
+            gt += key > K;
+            at += key == K && key != 0u;
+        }
+        gt = __reduce_add_sync(kFull, gt);
+        at = __reduce_add_sync(kFull, at);
+        if (lane == 0) {
+            s_gt[warp] = gt;
+            s_eq[warp] = at;
+        }
+        __syncthreads();
+        int pos = p0, eq = 0;
+        for (int w = 0; w < warp; ++w) {
+            pos += s_gt[w];
+            eq += s_eq[w];
+        }
+        if (cut) pos += eq < need ? eq : need;
+        pos = mcl_write(E, prm, K, need, cut, q0, q1, pos, p1, eq, col_out, val_out);
+        if (warp == kWarps - 1 && lane == 0 && pos != p1) set_status(ctl, ST_INTERNAL);
+        __syncthreads();
+        const double sum = block_sum(mcl_weights<kMclThreads>(val_out, p0, p1, threadIdx.x, prm.r), redd);
+        for (int q = p0 + (int)threadIdx.x; q < p1; q += kMclThreads)
+            val_out[q] = sum > 0.0 ? (float)(mcl_weight(val_out[q], prm.r) / sum) : 0.f;
+        // (s_gt and s_li are written again after the barriers of block_sum)
+    }
 }
 
 void launch_mcl_step(const spgemm_plan* p, const CsrDev& E, float theta, int k, double r,
@@ -312,13 +331,15 @@ void launch_mcl_step(const spgemm_plan* p, const CsrDev& E, float theta, int k, 
         return;
     }
     const MclParams prm{theta, k, r, order};
-    const int sms = p->num_sms;
+    const MclScratch ms{(unsigned*)w.row_scratch, w.row_scratch + E.rows, w.row_scratch + 2 * (size_t)E.rows};
+    const int grid = p->num_sms * 8, grid_long = p->num_sms * 6;
     int* counts = w.map;                       // E.rows ints of the workspace
-    SPG_LAUNCH(p, K_MCL, s, k_mcl_warp<false><<<sms * 8, kMclThreads, 0, s>>>(E, prm, counts, nullptr, nullptr, nullptr, w.ctl));
-    SPG_LAUNCH(p, K_MCL, s, k_mcl_block<false><<<sms, kMclBlockThreads, kMclStage * 4, s>>>(E, prm, counts, nullptr, nullptr, nullptr, w.ctl));
+    cudaMemsetAsync(w.ctl->work, 0, sizeof(w.ctl->work), s);
+    SPG_LAUNCH(p, K_MCL, s, k_mcl_select<<<grid, kMclThreads, 0, s>>>(E, prm, counts, ms, w.ctl));
+    SPG_LAUNCH(p, K_MCL, s, k_mcl_select_long<<<grid_long, kMclThreads, 0, s>>>(E, prm, counts, ms, w.ctl));
     launch_row_ptr(p, counts, E.rows, w, rpt_out, s);
-    SPG_LAUNCH(p, K_MCL, s, k_mcl_warp<true><<<sms * 8, kMclThreads, 0, s>>>(E, prm, counts, rpt_out, col_out, val_out, w.ctl));
-    SPG_LAUNCH(p, K_MCL, s, k_mcl_block<true><<<sms, kMclBlockThreads, kMclStage * 4, s>>>(E, prm, counts, rpt_out, col_out, val_out, w.ctl));
+    SPG_LAUNCH(p, K_MCL, s, k_mcl_write<<<grid, kMclThreads, 0, s>>>(E, prm, ms, rpt_out, col_out, val_out, w.ctl));
+    SPG_LAUNCH(p, K_MCL, s, k_mcl_write_long<<<grid_long, kMclThreads, 0, s>>>(E, prm, ms, rpt_out, col_out, val_out, w.ctl));
 }
 
 }  // namespace spg
