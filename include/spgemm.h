@@ -332,6 +332,11 @@ int spgemm_topk_dense(const spgemm_plan* plan, const float* X, int32_t n, int32_
 int spgemm_csr_scatter_dense(const spgemm_plan* plan, const spgemm_csr* M, const float* vals,
                              float* X, int64_t ldx, void* ws, size_t ws_bytes, void* stream);
 
+/* X = M as a dense matrix, zeros included (X is overwritten where the scatter
+ * above adds); arguments as for the scatter. Asynchronous. */
+int spgemm_csr_to_dense(const spgemm_plan* plan, const spgemm_csr* M, const float* vals, float* X,
+                        int64_t ldx, void* ws, size_t ws_bytes, void* stream);
+
 /* out[q] = D[i, j] for every entry q = (i, j) of M: a dense matrix read at
  * M's pattern (the gradient of A * TopK(X), dY * W^T, is needed only where
  * that product has entries). D: dense row-major M->rows x ldd (ldd >=

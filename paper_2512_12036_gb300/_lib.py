@@ -75,6 +75,7 @@ PROTOTYPES = {
     "spgemm_topk_dense": (ctypes.c_int, [c_vp, c_vp, c_i32, c_i32, c_i64, c_i32, c_vp, c_vp, c_vp,
                                          c_vp]),
     "spgemm_csr_scatter_dense": (ctypes.c_int, [c_vp, _CSR, c_vp, c_vp, c_i64, c_vp, c_sz, c_vp]),
+    "spgemm_csr_to_dense": (ctypes.c_int, [c_vp, _CSR, c_vp, c_vp, c_i64, c_vp, c_sz, c_vp]),
     "spgemm_csr_gather_dense": (ctypes.c_int, [c_vp, _CSR, c_vp, c_i64, c_vp, c_vp, c_sz, c_vp]),
     "spgemm_sample_rows": (ctypes.c_int, [c_vp, _CSR, c_i32, c_vp, c_i32, c_vp, c_sz, c_vp, c_vp,
                                           c_vp, _P(c_i64), c_vp]),

@@ -10,6 +10,7 @@ void occupancy_symbolic(spgemm_plan* p);
 void occupancy_numeric(spgemm_plan* p);
 void occupancy_bits(spgemm_plan* p);
 void occupancy_narrow(spgemm_plan* p);
+void occupancy_layer(spgemm_plan* p);
 void occupancy_backward(spgemm_plan* p);
 static size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
@@ -126,6 +127,7 @@ void init_occupancy(spgemm_plan* p) {
     occupancy_numeric(p);
     occupancy_bits(p);
     occupancy_narrow(p);
+    occupancy_layer(p);
     occupancy_backward(p);
 }
 
@@ -632,6 +634,25 @@ int spgemm_csr_scatter_dense(const spgemm_plan* plan, const spgemm_csr* M, const
     if (!ws || ws_bytes < sizeof(Ctl) || ((uintptr_t)ws & 255)) return SPGEMM_ERR_WORKSPACE;
     launch_scatter_dense(plan, dev_view(M), vals ? vals : M->vals, X, (long long)ldx, (Ctl*)ws,
                          (cudaStream_t)stream);
+    return cuda_err(cudaGetLastError());
+}
+
+int spgemm_csr_to_dense(const spgemm_plan* plan, const spgemm_csr* M, const float* vals, float* X,
+                        int64_t ldx, void* ws, size_t ws_bytes, void* stream) {
+    if (!plan) return SPGEMM_ERR_INVALID;
+    int rc = check_csr(M, vals == nullptr);
+    if (rc) return rc;
+    if (ldx < M->cols || (M->rows > 0 && M->cols > 0 && !X)) return SPGEMM_ERR_INVALID;
+    if (!ws || ws_bytes < sizeof(Ctl) || ((uintptr_t)ws & 255) != 0) return SPGEMM_ERR_WORKSPACE;
+    cudaStream_t s = (cudaStream_t)stream;
+    const CsrDev m = dev_view(M);
+    const float* v = vals ? vals : M->vals;
+    if (!launch_csr_to_dense(plan, m, v, X, (long long)ldx, (Ctl*)ws, s)) {
+        const cudaError_t e = cudaMemset2DAsync(X, sizeof(float) * (size_t)ldx, 0, sizeof(float) * (size_t)M->cols,
+                                                (size_t)M->rows, s);
+        if (e != cudaSuccess) return SPGEMM_ERR_CUDA;
+        launch_scatter_dense(plan, m, v, X, (long long)ldx, (Ctl*)ws, s);
+    }
     return cuda_err(cudaGetLastError());
 }
 

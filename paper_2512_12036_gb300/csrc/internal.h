@@ -282,6 +282,9 @@ void launch_topk(const spgemm_plan* p, const float* X, int n, int d, long long l
                  int* rpt, int* col, float* val, cudaStream_t s);
 void launch_scatter_dense(const spgemm_plan* p, const CsrDev& M, const float* vals, float* X,
                           long long ldx, Ctl* ctl, cudaStream_t s);
+// M as a dense matrix, zeros included; false (nothing done) for a wide M.
+bool launch_csr_to_dense(const spgemm_plan* p, const CsrDev& M, const float* vals, float* X,
+                         long long ldx, Ctl* ctl, cudaStream_t s);
 void launch_gather_dense(const spgemm_plan* p, const CsrDev& M, const float* D, long long ldd,
                          float* out, Ctl* ctl, cudaStream_t s);
 void launch_mcl_step(const spgemm_plan* p, const CsrDev& E, float theta, int k, double r,

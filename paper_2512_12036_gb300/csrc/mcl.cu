@@ -122,7 +122,13 @@ __global__ void __launch_bounds__(kMclThreads) k_mcl_select(CsrDev E, MclParams 
                 prefix |= (unsigned)dig << sh;
                 pmask |= 255u << sh;
                 above = run_at;
+                const int inside = hist[dig];
                 __syncwarp();
+                if (above + inside == prm.k) {                  // the whole bin is kept
+                    --prefix;
+                    above = prm.k;
+                    break;
+                }
             }
             K = prefix;
             need = prm.k - above;
@@ -141,7 +147,7 @@ __global__ void __launch_bounds__(kMclThreads) k_mcl_select_long(CsrDev E, MclPa
                                                                  MclScratch ms, Ctl* ctl) {
     __shared__ int red[33];
     __shared__ int hist[256];
-    __shared__ int s_li, s_dig, s_above;
+    __shared__ int s_li, s_dig, s_above, s_whole;
     __shared__ unsigned skey[kMclStage];
     const int nlong = ctl->work[0];
     for (;;) {
@@ -179,12 +185,18 @@ __global__ void __launch_bounds__(kMclThreads) k_mcl_select_long(CsrDev E, MclPa
                     if (threadIdx.x == 0) {
                         s_dig = dig;
                         s_above = run_at;
+                        s_whole = run_at + hist[dig] == prm.k;
                     }
                 }
                 __syncthreads();
                 prefix |= (unsigned)s_dig << sh;
                 pmask |= 255u << sh;
                 above = s_above;
+                if (s_whole) {                                  // the whole bin is kept
+                    --prefix;
+                    above = prm.k;
+                    break;
+                }
             }
         }
         if (threadIdx.x == 0) {

@@ -54,11 +54,15 @@ def scatter_dense(M: DeviceCSR, plan: Plan, vals: torch.Tensor | None = None,
                   out: torch.Tensor | None = None, ws: torch.Tensor | None = None,
                   stream=None) -> torch.Tensor:
     """out += M as a dense matrix (values ``vals`` on M's pattern if given)."""
-    if out is None:
-        out = torch.zeros(M.rows, M.cols, dtype=torch.float32, device=M.device)
     if ws is None:
         ws = _small_ws(plan, M.device)
     v = _ptr(vals) if vals is not None else None
+    if out is None:
+        out = torch.empty(M.rows, M.cols, dtype=torch.float32, device=M.device)
+        check(_lib.lib().spgemm_csr_to_dense(plan.handle, ctypes.byref(M.struct()), v, _ptr(out),
+                                             max(M.cols, 1), _ptr(ws), ws.numel(), _stream(stream)),
+              "spgemm_csr_to_dense")
+        return out
     check(_lib.lib().spgemm_csr_scatter_dense(plan.handle, ctypes.byref(M.struct()), v, _ptr(out),
                                               out.stride(0), _ptr(ws), ws.numel(),
                                               _stream(stream)),

@@ -174,3 +174,17 @@ def test_gcn_gin_sage_layers(plan):
     ss = (layers.layer_scales(np.eye(n), X, Ws, k, np.zeros((n, 32)))[0]
           + layers.layer_scales(dense_of(Am), X, Wn, k, np.zeros((n, 32)))[0])
     assert (np.abs(Ys - refs) <= (1e-5 + 48 * U + U) * ss + 1e-30).all()
+
+
+@pytest.mark.parametrize("cols", [1, 31, 33, 256, 2047, 2048, 2049, 5000])
+def test_scatter_into_a_new_matrix_writes_zeros_and_adds_repeats(plan, cols):
+    rng = np.random.default_rng(cols)
+    lens = rng.choice([0, 1, 31, 127, 128, 129, 300], size=60)
+    r = np.repeat(np.arange(lens.size), lens)
+    c = rng.integers(0, cols, size=r.size)
+    M = gen.csr_from_coo(lens.size, cols, r, c, rng.integers(-8, 9, size=r.size), sort=False)
+    want = np.zeros((lens.size, cols), np.float32)
+    np.add.at(want, (r, c), M.val)                      # small whole numbers: exact in any order
+    D = gnn.scatter_dense(DeviceCSR.from_host(M), plan)
+    torch.cuda.synchronize()
+    assert np.array_equal(D.cpu().numpy(), want)
