@@ -233,7 +233,7 @@ __device__ __forceinline__ int bin_of(const GroupArgs& g, int r, bool settle) {
     if (nnz <= o.block_max_nnz) return f64 ? NB_BLOCK64 : NB_BLOCK32;
     if (!f64 && nnz <= g.bits_cap) return NB_BITS32;
     const int L = log2_ceil_ll(ip);
-    return (f64 ? NB_DENSE64_0 : NB_DENSE32_0) + clampi(46 - L, 0, NB_DENSE_N - 1);
+    return (f64 ? NB_DENSE64_0 : NB_DENSE32_0) + clampi(kDenseTopLog - L, 0, NB_DENSE_N - 1);
 }
 
 __global__ void __launch_bounds__(kBinRows) k_group_hist(GroupArgs g, int nblk, int* blk_counts) {

@@ -114,6 +114,10 @@ enum : int {
     NB_SORT32A = 50, NB_SORT32B = 51, NB_SORT64A = 52, NB_SORT64B = 53
 };
 
+// accumulation dense bin q holds the rows of up to 2^(kDenseTopLog - q)
+// products (16 bins reach down to 2^14, below the lightest dense row)
+constexpr int kDenseTopLog = 29;
+
 // rows of the accumulation block tier that take the quarter- and half-size
 // table launches
 __host__ __device__ inline int block_small_nnz(const spgemm_opts& o) { return o.block_max_nnz / 4; }

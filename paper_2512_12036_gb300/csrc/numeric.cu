@@ -1386,13 +1386,13 @@ __global__ void __launch_bounds__(kHotThreads, 1) k_num_dense_hot(CsrDev A, CsrD
 // (popcounts of the cached bitmap), so the pieces need no merge step: they
 // are column-disjoint and already in order.
 // Column ranges per row when opts.dense_splits is 0: by the row's bin q
-// (bins of the fp64 tier hold rows with IP in (2^(45-q), 2^(46-q)]): one
+// (q: see kDenseTopLog): one
 // range per 128K intermediate products, at most 8 and at most one per panel.
 // (On the R-MAT scale 20 product, whose tier rows hold 1M-22M products, 8
 // ranges for every row measured best: 1 / 4 / 8 / 16 / 32 ranges gave 410 /
 // 262 / 249 / 252 / 269 ms; one range per 2M products gave 301 ms.)
 __device__ __forceinline__ int auto_splits(int q, int P) {
-    const int L = 46 - q;                     // IP <= 2^L
+    const int L = kDenseTopLog - q;           // IP <= 2^L
     const int sp = L >= 20 ? 8 : (L > 17 ? 1 << (L - 17) : 1);
     return sp < P ? sp : (P > 0 ? P : 1);
 }
