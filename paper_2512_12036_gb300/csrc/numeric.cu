@@ -852,6 +852,8 @@ constexpr int kRankPanels = 14;
 // products per lane per step of the value expansion: 4 / 5 / 6 -> 186.8 /
 // 183.9 / 181.1 ms at 12 panels, 7 -> 189.5 ms at 14
 constexpr int kRankUnroll = 6;
+constexpr int kRankRun = 6;           // steps of a run (2 / 3 / 4 / 6 -> 5,731 / 5,448 / 5,364 / 5,254 us
+                                      // on 1 in 32 rows, 5,486 without runs)
 constexpr int kRankOccUnroll = 8;     // occupancy expansion items are one int
 // A entries a row of this kernel may have (more go to k_num_dense<0>): the
 // fp32 rule keeps dense rows to at most fp32_max_terms (167 by default)
@@ -1074,7 +1076,7 @@ __global__ void __launch_bounds__(kRankThreads, kRankBlocks) k_num_dense_rank(Cs
                     if (i < cnt_sub && o < nnz_row) colC[out + o] = stage[i];
                     vals[i] = 0.f;
                 }
-                expand_tile_padded<kT, float, kRankUnroll>(tile, bs, len, mya, load, add);
+                expand_tile_padded<kT, float, kRankUnroll, false, kRankRun>(tile, bs, len, mya, load, add);
                 for (int i = t; i < cnt_sub; i += kT) {
                     const int o = written + rbase + i;
                     if (o < nnz_row) valC[out + o] = vals[i];
@@ -1415,6 +1417,8 @@ constexpr int kHotrStride = kHotrSlots + 1;   // copies of one slot in different
 #endif
 constexpr int kHotrThreads = SPG_HOTR_THREADS;
 constexpr int kHotrUnroll = SPG_HOTR_UNROLL;
+constexpr int kHotrRun = 3;           // steps of a run (1 / 2 / 3 / 4 -> 7,062 / 6,233 / 6,088 / 6,121 us on 1 in
+                                      // 32 rows, 6,175 without runs)
 static_assert(kHotrThreads / kHotCopies <= 160, "a copy must gather at most 160 terms per tile");
 
 __global__ void __launch_bounds__(kHotrThreads, 1) k_num_dense_hotr(
@@ -1642,7 +1646,7 @@ __global__ void __launch_bounds__(kHotrThreads, 1) k_num_dense_hotr(
                 nhs = hrp1 - h0 < kHotrSlots ? hrp1 - h0 : kHotrSlots;
                 cold = sub == 0;
                 if (cached) {
-                    expand_tile<kT, float, kHotrUnroll, true>(tile, bs, len, mya, load, apply);
+                    expand_tile<kT, float, kHotrUnroll, true, kHotrRun>(tile, bs, len, mya, load, apply);
                     fold();
                 } else {
                     for (int tb = rs; tb < re; tb += kT) {
@@ -1667,7 +1671,7 @@ __global__ void __launch_bounds__(kHotrThreads, 1) k_num_dense_hotr(
                                 set_status(ctl, ST_INVALID);
                             }
                         }
-                        expand_tile<kT, float, kHotrUnroll, true>(tile, tbs, tlen, a, load, apply);
+                        expand_tile<kT, float, kHotrUnroll, true, kHotrRun>(tile, tbs, tlen, a, load, apply);
                         fold();
                     }
                 }

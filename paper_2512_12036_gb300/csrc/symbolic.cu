@@ -14,6 +14,7 @@
 
 namespace spg {
 
+constexpr int kSymDenseRun = 8;      // steps of a run (3 / 4 / 6 / 8 -> 3,303 / 2,972 / 2,641 / 2,595 us)
 constexpr int kSymDenseUnroll = 6;   // products per warp step batch (4 / 6 / 8 -> 108.5 / 101.7 / 103.4 ms)
 constexpr int kSymBlockUnroll = 4;   // block hash tier (2 / 4 -> 11.8 / 11.2 ms)
 
@@ -360,7 +361,7 @@ __global__ void __launch_bounds__(kSymDenseThreads, 1) k_sym_dense(CsrDev A, Csr
             const int nw = (span + 31) >> 5;
             for (int q = threadIdx.x; q < nw; q += blockDim.x) bm[q] = 0u;
             __syncthreads();
-            block_expand<kSymDenseThreads, float, kSymDenseUnroll>(
+            block_expand<kSymDenseThreads, float, kSymDenseUnroll, kSymDenseRun>(
                 rs, re, tile,
                 [&](int j, int& bs, int& len, float&) { a_entry(A, B, j, bs, len, ctl); },
                 [&](int t) { return B.col[t]; },
