@@ -8,6 +8,7 @@ products (IP, Algorithm 1), allocation phase (symbolic), accumulation phase
 from __future__ import annotations
 
 import ctypes
+import itertools
 from dataclasses import dataclass
 
 import numpy as np
@@ -78,6 +79,28 @@ class DeviceCSR:
                          _ptr(self.val))
 
 
+# The allocation callback of spgemm(): one ctypes function for all calls (a new
+# one per call costs more than the call's arguments). ctx is the number under
+# which the call left its device; the tensors are put beside it.
+_calls: dict = {}
+_call_ids = itertools.count(1)
+
+
+def _alloc_result(ctx, nnz, colp, valp):
+    call = _calls[ctx]
+    try:
+        call.append(torch.empty(int(nnz), dtype=torch.int32, device=call[0]))
+        call.append(torch.empty(int(nnz), dtype=torch.float32, device=call[0]))
+    except RuntimeError:                       # out of memory: the call returns SPGEMM_ERR_BUDGET
+        return 1
+    colp[0] = _ptr(call[1])
+    valp[0] = _ptr(call[2])
+    return 0
+
+
+_ALLOC_RESULT = _lib.ALLOC_FN(_alloc_result)
+
+
 def default_opts() -> dict:
     o = OptsStruct()
     check(_lib.lib().spgemm_opts_default(ctypes.byref(o)), "spgemm_opts_default")
@@ -119,15 +142,27 @@ class Plan:
 
     def workspace(self, A: DeviceCSR, B: DeviceCSR, stream=None) -> torch.Tensor:
         """A 256-byte aligned, initialised workspace for operands of these shapes."""
-        ws = self._workspace_buffer(A, B)
+        ws = self._buffer(self.workspace_bytes(A, B), A.device)
         self.workspace_init(ws, stream)
         return ws
 
-    def _workspace_buffer(self, A: DeviceCSR, B: DeviceCSR) -> torch.Tensor:
-        nbytes = self.workspace_bytes(A, B)
-        ws = torch.empty(nbytes + 256, dtype=torch.uint8, device=A.device)
-        off = (-ws.data_ptr()) % 256
-        return ws[off:off + nbytes]
+    def workspace_for_rows(self, rows: int, device, stream=None) -> torch.Tensor:
+        """An initialised workspace for the steps that take one matrix of
+        ``rows`` rows (clustering step, sampling, column selection)."""
+        n = ctypes.c_size_t()
+        one, none = CsrStruct(rows, 0, 0, None, None, None), CsrStruct(0, 0, 0, None, None, None)
+        check(_lib.lib().spgemm_workspace_bytes(self.handle, ctypes.byref(one), ctypes.byref(none),
+                                                ctypes.byref(n)), "spgemm_workspace_bytes")
+        ws = self._buffer(int(n.value), device)
+        self.workspace_init(ws, stream)
+        return ws
+
+    @staticmethod
+    def _buffer(nbytes: int, device) -> torch.Tensor:
+        """``nbytes`` from a 256-byte boundary on."""
+        buf = torch.empty(nbytes + 256, dtype=torch.uint8, device=device)
+        off = (-buf.data_ptr()) % 256
+        return buf[off:off + nbytes]
 
     def workspace_init(self, ws: torch.Tensor, stream=None) -> None:
         check(_lib.lib().spgemm_workspace_init(self.handle, _ptr(ws), ws.numel(), _stream(stream)),
@@ -287,29 +322,31 @@ class Plan:
         """C = A*B through the one-call entry point (C allocated by torch).
         ``ip_row`` (int64, A.rows, on the device) receives the per-row
         intermediate-product counts of the call (Algorithm 1) when given."""
+        L, dev, m = _lib.lib(), A.device, A.rows
+        sA, sB = A.struct(), B.struct()
+        # workspace and scratch from one buffer (the call initialises them)
+        size = ctypes.c_size_t()
         if ws is None:
-            ws = self._workspace_buffer(A, B)      # (the call initialises it)
-        dev = A.device
-        if ip_row is None:
-            ip_row = torch.empty(A.rows, dtype=torch.int64, device=dev)
-        row_nnz = torch.empty(A.rows, dtype=torch.int32, device=dev)
-        row_ptr = torch.empty(A.rows + 1, dtype=torch.int32, device=dev)
-        keep = {}
-
-        def alloc(ctx, nnz, colp, valp):
-            keep["col"] = torch.empty(int(nnz), dtype=torch.int32, device=dev)
-            keep["val"] = torch.empty(int(nnz), dtype=torch.float32, device=dev)
-            colp[0] = _ptr(keep["col"])
-            valp[0] = _ptr(keep["val"])
-            return 0
-
-        cb = _lib.ALLOC_FN(alloc)
+            check(L.spgemm_workspace_bytes(self.handle, ctypes.byref(sA), ctypes.byref(sB),
+                                           ctypes.byref(size)), "spgemm_workspace_bytes")
+        wsn = (size.value + 255) // 256 * 256 if ws is None else 0
+        buf = torch.empty(wsn + (0 if ip_row is not None else 8 * m) + 4 * m + 512, dtype=torch.uint8,
+                          device=dev)
+        at = buf.data_ptr() + (-buf.data_ptr()) % 256
+        ws_ptr, ws_bytes = (at, size.value) if ws is None else (_ptr(ws), ws.numel())
+        ip_ptr = at + wsn if ip_row is None else _ptr(ip_row)
+        nnz_ptr = at + wsn + (8 * m if ip_row is None else 0)
+        row_ptr = torch.empty(m + 1, dtype=torch.int32, device=dev)
         nnz = ctypes.c_int64()
-        check(_lib.lib().spgemm(self.handle, ctypes.byref(A.struct()), ctypes.byref(B.struct()),
-                                _ptr(ws), ws.numel(), _ptr(ip_row), _ptr(row_nnz), _ptr(row_ptr),
-                                cb, None, ctypes.byref(nnz), _stream(stream)),
-              "spgemm")
-        return DeviceCSR(A.rows, B.cols, row_ptr, keep["col"], keep["val"])
+        ctx = next(_call_ids)
+        call = _calls[ctx] = [dev]
+        try:
+            check(L.spgemm(self.handle, ctypes.byref(sA), ctypes.byref(sB), ws_ptr, ws_bytes, ip_ptr,
+                           nnz_ptr, row_ptr.data_ptr(), _ALLOC_RESULT, ctx, ctypes.byref(nnz),
+                           _stream(stream)), "spgemm")
+        finally:
+            del _calls[ctx]
+        return DeviceCSR(m, B.cols, row_ptr, call[1], call[2])
 
     def spgemm_blocks(self, A: DeviceCSR, B: DeviceCSR, max_block_nnz: int = 2**31 - 1,
                       ws: torch.Tensor | None = None, stream=None, out=None):

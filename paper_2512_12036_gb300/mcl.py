@@ -21,8 +21,7 @@ def mcl_step(plan: Plan, E: DeviceCSR, theta: float, k: int, r: float, order: in
              ws: torch.Tensor | None = None, stream=None) -> DeviceCSR:
     """Prune (< theta), keep the top k per row, inflate (^r), normalise rows."""
     if ws is None:
-        ws = plan.workspace(E, DeviceCSR(0, 0, torch.zeros(1, dtype=torch.int32, device=E.device),
-                                         torch.zeros(0, dtype=torch.int32, device=E.device), None))
+        ws = plan.workspace_for_rows(E.rows, E.device)
     cap = E.nnz if k < 0 else min(E.nnz, E.rows * k)
     rp = torch.empty(E.rows + 1, dtype=torch.int32, device=E.device)
     col = torch.empty(max(cap, 1), dtype=torch.int32, device=E.device)

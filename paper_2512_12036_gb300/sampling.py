@@ -28,21 +28,12 @@ from .api import DeviceCSR, Plan, _ptr, _stream
 UNIFORM, BY_VALUE, BY_SQUARE = 0, 1, 2
 
 
-def _ws_rows(plan: Plan, rows: int, device) -> torch.Tensor:
-    """Workspace for a matrix of ``rows`` rows (status word, scan scratch)."""
-    empty = DeviceCSR(rows, 0, torch.zeros(rows + 1, dtype=torch.int32, device=device),
-                      torch.zeros(0, dtype=torch.int32, device=device),
-                      torch.zeros(0, dtype=torch.float32, device=device))
-    return plan.workspace(empty, DeviceCSR(0, 0, torch.zeros(1, dtype=torch.int32, device=device),
-                                           empty.col, empty.val))
-
-
 def sample_rows(P: DeviceCSR, s: int, u: torch.Tensor, mode: int, plan: Plan,
                 stream=None) -> DeviceCSR:
     """SAMPLE: up to s distinct columns per row of P drawn with uniforms u
     (P.rows x s, fp32 in [0, 1)); value 1 at every drawn column."""
     dev = P.device
-    ws = _ws_rows(plan, P.rows, dev)
+    ws = plan.workspace_for_rows(P.rows, dev)
     rp = torch.empty(P.rows + 1, dtype=torch.int32, device=dev)
     col = torch.empty(P.rows * s, dtype=torch.int32, device=dev)
     val = torch.empty(P.rows * s, dtype=torch.float32, device=dev)
@@ -60,7 +51,7 @@ def select_columns(Q: DeviceCSR, plan: Plan, stream=None) -> tuple[DeviceCSR, De
     dev = Q.device
     n = Q.cols
     cap = max(1, min(n, Q.nnz))
-    ws = _ws_rows(plan, n, dev)
+    ws = plan.workspace_for_rows(n, dev)
     S_rp = torch.empty(n + 1, dtype=torch.int32, device=dev)
     F_rp = torch.empty(cap + 1, dtype=torch.int32, device=dev)
     S_col = torch.empty(cap, dtype=torch.int32, device=dev)
