@@ -80,6 +80,12 @@ WsLayout ws_layout(const spgemm_plan* p, long long m, long long b_rows, long lon
             }
         }
     }
+    // (rows with cached bitmaps have their panels' counts instead)
+    if (L.rc_nslots == 0 && L.has_hot && m > 0 && b_cols > p->opts.block_max_nnz && L.panels >= 2 &&
+        L.panels <= kMaxPanels) {
+        L.part_nnz = off;
+        off = align256(off + sizeof(int) * kParts * (size_t)m);
+    }
     L.total = off;
     return L;
 }
@@ -105,6 +111,7 @@ WsPtrs ws_ptrs(const WsLayout& L, void* ws, int panel_cols) {
     w.rc_pc = L.rc_nslots > 0 && L.rc_pc > 0 ? (int*)(b + L.rc_pc) : nullptr;
     w.rc_nslots = L.rc_nslots;
     w.rc_wpr = L.rc_wpr;
+    w.part_nnz = L.part_nnz > 0 ? (int*)(b + L.part_nnz) : nullptr;
     w.nb_bits = L.nc_bits > 0 ? (unsigned*)(b + L.nb_bits) : nullptr;
     w.nc_bits = L.nc_bits > 0 ? (unsigned*)(b + L.nc_bits) : nullptr;
     w.nblk = L.nblk;

@@ -88,6 +88,7 @@ constexpr int kBlockThreadsFull = 1024;   // block tiers' full-size-table launch
 // expansion tile); rows with more take the dense-array fallback kernel
 constexpr int kRankTileEntries = 256;
 constexpr int kNumDenseThreads = 1024;
+constexpr int kParts = 8;           // column ranges whose entries the allocation bitmap tier counts per row
 constexpr int kMaxPanels = 1024;    // above this the heavy path filters whole B rows
 
 // Bins (phase-specific meaning). Allocation phase:
@@ -165,6 +166,7 @@ struct WsLayout {
     size_t rc_bits = 0;      // u32 [rc_nslots][rc_wpr] row bitmaps of the allocation phase
     size_t rc_pc = 0;        // int [rc_nslots][panels] entries of each table panel of a cached row
     int rc_nslots = 0, rc_wpr = 0;
+    size_t part_nnz = 0;     // int32 [m][kParts] entries of a heavy row by column range
     size_t nb_bits = 0;      // u32 [B.rows][nw] bitmaps of B's rows, nw = ceil(B.cols / 32)
     size_t nc_bits = 0;      // u32 [m][nw]       and of C's rows (narrow tiers; B.cols <= kNarrowCols)
     bool has_hot = false;
@@ -192,6 +194,7 @@ struct WsPtrs {
     unsigned* rc_bits;
     int* rc_pc;              // per-panel entry counts of the cached rows, or nullptr
     int rc_nslots, rc_wpr;
+    int* part_nnz;           // nullptr: not counted
     unsigned* nb_bits;       // narrow tiers' bitmaps, or nullptr
     unsigned* nc_bits;
     int nblk, nscan, panels, panel_cols;
@@ -229,6 +232,8 @@ void launch_group(const spgemm_plan* p, const GroupArgs& g, const WsPtrs& w, int
 void launch_row_ptr(const spgemm_plan* p, const int* row_nnz, int n, const WsPtrs& w,
                     int* row_ptr, cudaStream_t s);
 
+// Columns that the allocation bitmap tier takes in one pass.
+long long sym_dense_span(const spgemm_plan* p);
 void launch_symbolic(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const long long* ip,
                      const WsPtrs& w, int* row_nnz, cudaStream_t s);
 void launch_check_rpt(const spgemm_plan* p, const CsrDev& M, const WsPtrs& w, cudaStream_t s);

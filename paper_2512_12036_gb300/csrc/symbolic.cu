@@ -337,7 +337,8 @@ __global__ void __launch_bounds__(kSymDenseThreads, 1) k_sym_dense(CsrDev A, Csr
                                                                 int nwords, int* rc_slot,
                                                                 unsigned* rc_bits, int rc_nslots,
                                                                 int rc_wpr, int cache_min,
-                                                                int* rc_pc, int P, int wpp) {
+                                                                int* rc_pc, int P, int wpp,
+                                                                int* part_nnz) {
     extern __shared__ unsigned bm[];
     __shared__ int s_idx, s_slot;
     __shared__ int red[33];
@@ -373,9 +374,10 @@ __global__ void __launch_bounds__(kSymDenseThreads, 1) k_sym_dense(CsrDev A, Csr
                     else key_ok(key, B, ctl);
                 });
             int cnt = 0;
-            // one-pass rows with a cache: the count by table panel (a warp
-            // per panel), kept for the accumulation phase's pass offsets
-            const bool by_panel = rc_pc != nullptr && c0l == 0 && B.cols <= span_max && P <= kMaxPanels;
+            // one-pass rows: the count by table panel (a warp per panel), kept
+            // for the accumulation phase's pass offsets, or summed to parts
+            const bool by_panel = (rc_pc != nullptr || part_nnz != nullptr) && c0l == 0 &&
+                                  B.cols <= span_max && P <= kMaxPanels;
             if (by_panel) {
                 const int lane = lane_id(), nwarp = blockDim.x >> 5;
                 for (int p = threadIdx.x >> 5; p < P; p += nwarp) {
@@ -393,6 +395,12 @@ __global__ void __launch_bounds__(kSymDenseThreads, 1) k_sym_dense(CsrDev A, Csr
             }
             nnz += block_sum(cnt, red);
             // (block_sum ends with a barrier: bm and s_pc are final here)
+            if (part_nnz != nullptr && by_panel && threadIdx.x < kParts) {
+                const int g = threadIdx.x;
+                int c = 0;
+                for (int p = P * g / kParts; p < P * (g + 1) / kParts; ++p) c += s_pc[p];
+                part_nnz[(size_t)row * kParts + g] = c;
+            }
             if (rc_slot != nullptr && c0l == 0 && B.cols <= span_max && nnz > cache_min &&
                 nw == rc_wpr) {
                 if (threadIdx.x == 0) {
@@ -446,6 +454,8 @@ static size_t sym_dense_smem(const spgemm_plan* p) {
     if (words > cap) words = cap;
     return words * 4;
 }
+
+long long sym_dense_span(const spgemm_plan* p) { return (long long)sym_dense_smem(p) / 4 * 32; }
 
 static size_t staged_smem() { return sizeof(int) * 4 * (size_t)kStageMax; }
 
@@ -579,7 +589,7 @@ void launch_symbolic(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, con
                k_sym_dense<<<sms * p->occ_sym_dense, kSymDenseThreads, sd, s>>>(
                    A, B, w.map, w.ctl, row_nnz, SB_DENSE0, SB_DENSE0 + SB_DENSE_N, 1, (int)(sd / 4),
                    w.rc_slot, w.rc_bits, w.rc_nslots, w.rc_wpr, p->opts.block_max_nnz, w.rc_pc,
-                   w.panels, w.panel_cols / 32));
+                   w.panels, w.panel_cols / 32, w.part_nnz));
 }
 
 }  // namespace spg

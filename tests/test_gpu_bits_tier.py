@@ -41,3 +41,29 @@ def test_rows_at_tile_and_class_edges(cols, messy):
         C = Plan(**opts).spgemm(dA, dB)
         torch.cuda.synchronize()
         compare(C.to_host(), ref)
+
+
+@pytest.mark.parametrize("cols,panel", [(300_000, 16384), (300_000, 4096), (40_000, 1024), (1_200_000, 16384)])
+@pytest.mark.parametrize("repeats", [False, True])
+def test_few_heavy_rows_cut_into_column_ranges(cols, panel, repeats):
+    # a handful of fp64-bound rows of 2^15 to 2^20 products: the lightest in
+    # one range, the heaviest in as many as the columns allow
+    rng = np.random.default_rng(cols + panel + repeats)
+    lens = rng.integers(100, 500, size=3000)
+    r = np.repeat(np.arange(lens.size), lens)
+    c = np.concatenate([np.sort(rng.choice(cols, size=n, replace=False)) for n in lens])
+    c[::97] = rng.integers(0, 50, size=c[::97].size)                # hot columns
+    key = np.unique(r * np.int64(cols) + c)
+    r, c = key // cols, key % cols
+    if repeats:
+        r, c = np.concatenate([r, r[::50]]), np.concatenate([c, c[::50]])
+    B = gen.csr_from_coo(lens.size, cols, r, c, gen.uniform_open_closed(rng, r.size))
+    na = [170, 400, 900, 1100, 2000, 3000]
+    ra = np.repeat(np.arange(len(na)), na)
+    ca = np.concatenate([rng.choice(lens.size, size=n, replace=False) for n in na])
+    A = gen.csr_from_coo(len(na), lens.size, ra, ca, gen.uniform_open_closed(rng, ra.size))
+    ip, _ = oracle.ip_count(A, B)
+    assert ip.min() < 1 << 17 and ip.max() > 1 << 19
+    C = Plan(panel_cols=panel).spgemm(DeviceCSR.from_host(A), DeviceCSR.from_host(B))
+    torch.cuda.synchronize()
+    compare(C.to_host(), oracle.spgemm(A, B))
