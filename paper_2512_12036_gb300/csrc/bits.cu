@@ -15,7 +15,8 @@ namespace spg {
 
 constexpr int kBitsUnroll = 2;    // products per lane in flight in a walk
 constexpr int kBitsRun = 4;       // steps of a run (1 / 2 / 3 / 4 -> 1,712 / 1,310 / 1,225 / 1,211 us for the four
-                                  // kernels of R-MAT 2^15 squared)
+                                  // kernels of R-MAT 2^15 squared); none in the value walk of the sparser
+                                  // rows, whose segments are shorter (1,616 -> 1,600 us, 1,075 products a row)
 
 // One tile of A entries: non-empty segments, their offsets and multipliers.
 template <int kE>
@@ -85,11 +86,11 @@ __device__ __forceinline__ int bits_fill(BitsTile<kE>& tile, const CsrDev& A, co
     return n;
 }
 
-template <int kT, int kE, class Load, class Apply>
+template <int kT, int kE, int kRun = kBitsRun, class Load, class Apply>
 __device__ __forceinline__ void bits_walk(const BitsTile<kE>& tile, int n, long long products,
                                           Load&& load, Apply&& apply) {
     if (products < (1ll << 30)) {
-        expand_walk<int, kT / 32, float, kBitsUnroll, false, kBitsRun>(tile.off, tile.bs, tile.a, n,
+        expand_walk<int, kT / 32, float, kBitsUnroll, false, kRun>(tile.off, tile.bs, tile.a, n,
                                                              (int)products, load, apply);
         return;
     }
@@ -256,12 +257,12 @@ __global__ void __launch_bounds__(kT, 1024 / kT) k_num_bits(CsrDev A, CsrDev B, 
             }
         };
         if (re - rs <= kE) {                       // the tile of the first walk is the whole row
-            bits_walk<kT, kE>(tile, n, products, load, apply);
+            bits_walk<kT, kE, kCols ? 0 : kBitsRun>(tile, n, products, load, apply);
             __syncthreads();
         } else {
             for (int j0 = rs; j0 < re; j0 += kE) {
                 n = bits_fill<kT, kE>(tile, A, B, j0, re, true, ctl, products);
-                bits_walk<kT, kE>(tile, n, products, load, apply);
+                bits_walk<kT, kE, kCols ? 0 : kBitsRun>(tile, n, products, load, apply);
                 __syncthreads();
             }
         }

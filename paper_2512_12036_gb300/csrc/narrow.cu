@@ -19,7 +19,7 @@
 namespace spg {
 
 constexpr int kNarrowThreads = 256;
-constexpr int kNarrowUnroll = 4;     // A entries whose products are in flight
+constexpr int kNarrowUnroll = 4;     // A entries whose products are in flight (2 / 4 / 8 -> 943 / 738 / 892 us)
 
 // Bitmaps of B's rows (nw words each); a row that repeats a column sets
 // ctl->narrow_dup. Four rows are in flight per warp: the row pointers of 32
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kNarrowThreads) k_sym_narrow(CsrDev A, CsrDev 
 // What bounds it: instruction issue and the shared-memory round trip of every
 // A entry. 589,000 rows of 612 products over 256 columns: 2,013 us with
 // atomics, a bitmap marked per product and each lane emitting its own word (8
-// of 32 lanes, scattered stores), 768 us now.
+// of 32 lanes, scattered stores), 738 us now.
 template <typename Acc>
 __global__ void __launch_bounds__(kNarrowMaxWarps * 32) k_num_narrow(CsrDev A, CsrDev B,
                                                                      const int* map, Ctl* ctl,
@@ -214,6 +214,14 @@ __global__ void __launch_bounds__(kNarrowMaxWarps * 32) k_num_narrow(CsrDev A, C
                         c[u] = B.col[qs[u] + lane];
                         v[u] = B.val[qs[u] + lane];
                     }
+                }
+                if (most <= 32) {                            // warp-uniform: no loops
+#pragma unroll
+                    for (int u = 0; u < kNarrowUnroll; ++u) {
+                        if ((unsigned)c[u] < (unsigned)B.cols) dense[c[u]] += (Acc)qa[u] * (Acc)v[u];
+                        __syncwarp();
+                    }
+                    continue;
                 }
 #pragma unroll
                 for (int u = 0; u < kNarrowUnroll; ++u) {
