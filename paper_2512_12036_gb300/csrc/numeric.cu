@@ -1306,9 +1306,17 @@ __global__ void __launch_bounds__(kHotThreads, 1) k_num_dense_hot(CsrDev A, CsrD
         int written = 0, upto = nnz_row;
         if (q1 - q0 < kParts) {
             const int* parts = part_nnz + (size_t)row * kParts;
-            for (int q = 0; q < q0; ++q) written += parts[q];
-            upto = written;
-            for (int q = q0; q < q1; ++q) upto += parts[q];
+            bool ok = true;
+            upto = 0;
+            for (int q = 0; q < q1 && ok; ++q) {
+                if (q == q0) written = upto;
+                ok = parts[q] >= 0 && parts[q] <= nnz_row - upto;
+                if (ok) upto += parts[q];
+            }
+            if (!ok) {                                   // not this row's counts: write nothing
+                set_status(ctl, ST_INTERNAL);
+                continue;
+            }
         }
         for (int pass = 0; pass < npass; ++pass) {
             const int p0 = gp0 + pass * ppp;

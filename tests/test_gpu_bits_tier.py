@@ -67,3 +67,32 @@ def test_few_heavy_rows_cut_into_column_ranges(cols, panel, repeats):
     C = Plan(panel_cols=panel).spgemm(DeviceCSR.from_host(A), DeviceCSR.from_host(B))
     torch.cuda.synchronize()
     compare(C.to_host(), oracle.spgemm(A, B))
+
+
+def test_part_counts_of_another_call_are_reported():
+    # rows cut into column ranges read their parts' counts from the workspace
+    # (its last array): counts that cannot be theirs set the status word, and
+    # nothing is written outside the rows
+    from paper_2512_12036_gb300 import SpgemmError
+    rng = np.random.default_rng(3)
+    cols, k = 300_000, 3000
+    rb = np.repeat(np.arange(k), 300)
+    B = gen.csr_from_coo(k, cols, rb, rng.integers(0, cols, size=rb.size), gen.uniform_open_closed(rng, rb.size))
+    na = [1100, 2000, 2900]
+    ra = np.repeat(np.arange(len(na)), na)
+    ca = np.concatenate([rng.choice(k, size=n, replace=False) for n in na])
+    A = gen.csr_from_coo(len(na), k, ra, ca, gen.uniform_open_closed(rng, ra.size))
+    plan, dA, dB = Plan(), DeviceCSR.from_host(A), DeviceCSR.from_host(B)
+    for fill in (-5, 0x7fffffff):
+        ws = plan.workspace(dA, dB)
+        ip_row, _ = plan.count(dA, dB, ws)
+        row_nnz, nnz = plan.symbolic(dA, dB, ip_row, ws)
+        rp, _ = plan.row_ptr(row_nnz, ws)
+        ws[-256:].view(torch.int32).fill_(fill)
+        buf = torch.full((2, nnz + 2048), -7, dtype=torch.int32, device="cuda")
+        col, val = buf[0, 1024:1024 + nnz], buf[1, 1024:1024 + nnz].view(torch.float32)
+        plan.numeric(dA, dB, ip_row, rp, ws, col, val)
+        torch.cuda.synchronize()
+        assert (buf[:, :1024] == -7).all() and (buf[:, 1024 + nnz:] == -7).all()
+        with pytest.raises(SpgemmError):
+            plan.check_status(ws, "stale part counts")
