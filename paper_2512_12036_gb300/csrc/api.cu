@@ -53,11 +53,14 @@ WsLayout ws_layout(const spgemm_plan* p, long long m, long long b_rows, long lon
         off = align256(off + 8 * (size_t)b_nnz);
     }
     const long long wpr = (b_cols + 31) / 32;
-    if (b_nnz > 0 && wpr > 0 && b_cols <= kNarrowCols && m > 0) {
-        L.nb_bits = off;
-        off = align256(off + sizeof(unsigned) * (size_t)wpr * (size_t)b_rows);
-        L.nc_bits = off;
-        off = align256(off + sizeof(unsigned) * (size_t)wpr * (size_t)m);
+    // narrow tiers' bitmaps: in the place of the dense tiers' tables, which a
+    // B of so few columns never has, when they fit there
+    if (L.has_hot && m > 0 && b_cols <= kNarrowCols && b_cols <= p->opts.block_max_nnz) {
+        const size_t nb = L.bpanel, nc = align256(nb + sizeof(unsigned) * (size_t)wpr * (size_t)b_rows);
+        if (nc + sizeof(unsigned) * (size_t)wpr * (size_t)m <= off) {
+            L.nb_bits = nb;
+            L.nc_bits = nc;
+        }
     }
     if (p->opts.row_cache_mb > 0 && m > 0 && wpr > 0 && wpr <= kRowCacheMaxWords) {
         const size_t bytes = (size_t)p->opts.row_cache_mb << 20;

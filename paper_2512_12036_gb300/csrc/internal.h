@@ -167,8 +167,8 @@ struct WsLayout {
     size_t rc_pc = 0;        // int [rc_nslots][panels] entries of each table panel of a cached row
     int rc_nslots = 0, rc_wpr = 0;
     size_t part_nnz = 0;     // int32 [m][kParts] entries of a heavy row by column range
-    size_t nb_bits = 0;      // u32 [B.rows][nw] bitmaps of B's rows, nw = ceil(B.cols / 32)
-    size_t nc_bits = 0;      // u32 [m][nw]       and of C's rows (narrow tiers; B.cols <= kNarrowCols)
+    size_t nb_bits = 0;      // u32 [B.rows][nw] bitmaps of B's rows, nw = ceil(B.cols / 32), and
+    size_t nc_bits = 0;      // u32 [m][nw]       of C's (narrow tiers; 0: no room for them)
     bool has_hot = false;
     size_t total = 0;
     int m = 0, nblk = 0, nscan = 0, panels = 0;

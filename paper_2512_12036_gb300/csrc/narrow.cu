@@ -6,8 +6,10 @@
 // when A has enough entries to pay for it B's rows are first turned into
 // bitmaps (one pass over B's columns) and a row of C is the OR of one bitmap
 // per A entry: 32 bytes an entry at 256 columns where the products' columns
-// are 4 bytes each. Otherwise the products are marked one by one. Either way
-// C's bitmap is kept for the accumulation phase.
+// are 4 bytes each. Otherwise the products are marked one by one. C's bitmap is
+// kept for the accumulation phase where the workspace has room for it (the
+// place of the dense tiers' tables, 20 bytes per entry of B); without it that
+// phase marks a row's products again.
 //
 // Accumulation phase: a dense accumulator over B's columns per warp. A B row
 // without a repeated column touches every accumulator at most once, so its
@@ -139,7 +141,7 @@ __global__ void __launch_bounds__(kNarrowThreads) k_sym_narrow(CsrDev A, CsrDev 
         const unsigned word = bm[lane];
         bm[lane] = 0u;
         const int nnz = __reduce_add_sync(kFull, __popc(word));
-        if (lane < nw) cbits[(long long)row * nw + lane] = word;
+        if (cbits != nullptr && lane < nw) cbits[(long long)row * nw + lane] = word;
         if (lane == 0) row_nnz[row] = nnz;
         __syncwarp();
     }
@@ -158,6 +160,9 @@ __global__ void __launch_bounds__(kNarrowMaxWarps * 32) k_num_narrow(CsrDev A, C
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int warp = threadIdx.x >> 5, lane = lane_id();
     Acc* dense = reinterpret_cast<Acc*>(sm_raw) + warp * nw * 32;
+    __shared__ unsigned s_bm[kNarrowMaxWarps][32];      // without C's bitmaps
+    unsigned* bm = s_bm[warp];
+    bm[lane] = 0u;
     for (int c = lane; c < nw * 32; c += 32) dense[c] = Acc(0);
     __syncwarp();
     const int begin = ctl->bin_off[bin], end = ctl->bin_off[bin + 1];
@@ -172,9 +177,21 @@ __global__ void __launch_bounds__(kNarrowMaxWarps * 32) k_num_narrow(CsrDev A, C
         const int row = row_begin + r;
         const int out = rptC[r];
         const int nnz_row = rptC[r + 1] - out;
-        const unsigned word = lane < nw ? cbits[(long long)row * nw + lane] : 0u;
         int rs, re;
         row_extent(A, row, rs, re, ctl);
+        unsigned word = 0u;
+        if (cbits != nullptr) {
+            if (lane < nw) word = cbits[(long long)row * nw + lane];
+        } else {
+            warp_expand_ahead<kWarpAhead, false>(
+                A, B, rs, re, ctl, [&](int t) { return B.col[t]; },
+                [&](int c, float, unsigned) {
+                    if ((unsigned)c < (unsigned)B.cols) atomicOr(&bm[c >> 5], 1u << (c & 31));
+                });
+            __syncwarp();
+            word = bm[lane];
+            bm[lane] = 0u;
+        }
         for (int base = rs; base < re; base += 32) {
             const int j = base + lane;
             int bs = 0, len = 0;
@@ -268,12 +285,11 @@ __global__ void k_narrow_reset(Ctl* ctl, int dup) { ctl->narrow_dup = dup; }
 
 void launch_sym_narrow(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const WsPtrs& w,
                        int* row_nnz, cudaStream_t s) {
-    if (!w.nb_bits) return;
     const int nw = (B.cols + 31) / 32;
     const int grid = p->num_sms * 8;
     // B's bitmaps cost a pass over B and save a pass over the products: worth
     // it unless A selects few of B's rows (B rows are then read about once)
-    const bool build = A.nnz >= B.rows / 2;
+    const bool build = w.nc_bits != nullptr && A.nnz >= B.rows / 2;
     SPG_LAUNCH(p, K_SYM_NARROW, s, k_narrow_reset<<<1, 1, 0, s>>>(w.ctl, build ? 0 : 1));
     if (build) {
         SPG_LAUNCH(p, K_SYM_NARROW, s, k_narrow_build<<<grid, kNarrowThreads, 0, s>>>(B, nw, w.nb_bits, w.ctl));
@@ -291,7 +307,6 @@ void launch_sym_narrow(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, c
 
 void launch_num_narrow(const spgemm_plan* p, bool f64, const CsrDev& A, const CsrDev& B, const WsPtrs& w,
                        const int* rptC, int row_begin, int* colC, float* valC, cudaStream_t s) {
-    if (!w.nc_bits) return;
     const int nw = (B.cols + 31) / 32;
     const int nwp = narrow_warps(p);
     const int grid = p->num_sms * (64 / nwp > 1 ? 64 / nwp : 1);

@@ -247,14 +247,25 @@ def gpu_server(slots: int = 4, budget_bytes: int = 64 << 30, device: int = 0,
 
     def bound_fn(req):
         torch.cuda.set_device(device)
+        A, B = req.A, req.B
         count_arena.reset()
-        nws = count_plan.workspace_bytes(req.A, req.B)
+        nws = count_plan.workspace_bytes(A, B)
         with torch.cuda.stream(count_stream):
-            ws = count_arena.take(nws, torch.uint8)
+            ip_row = count_arena.take(8 * max(A.rows, 1), torch.int64)[:A.rows]
+            # counted in one go, or by as many rows as the arena holds a
+            # workspace for
+            step, need = A.rows, nws
+            while need > count_arena.free() and step > 1:
+                step = (step + 1) // 2
+                need = count_plan.workspace_bytes(A.view_rows(0, step), B)
+            ws = count_arena.take(need, torch.uint8)
             count_plan.workspace_init(ws)
-            ip_row = count_arena.take(8 * max(req.A.rows, 1), torch.int64)[:req.A.rows]
-            ip_row, ip_total = count_plan.count(req.A, req.B, ws, ip_row=ip_row)
-            bound = request_bound(count_plan, req.A, req.B, nws, ip_total)
+            ip_total = 0
+            for r0 in range(0, max(A.rows, 1), max(step, 1)):
+                r1 = min(r0 + step, A.rows)
+                _, part = count_plan.count(A.view_rows(r0, r1), B, ws, ip_row=ip_row[r0:r1])
+                ip_total += part
+            bound = request_bound(count_plan, A, B, nws, ip_total)
             # the per-row counts are needed only to split a request that does
             # not fit a slot; they go to host memory (on the count stream,
             # before the next request reuses the arena), never to a new
@@ -266,7 +277,9 @@ def gpu_server(slots: int = 4, budget_bytes: int = 64 << 30, device: int = 0,
         """Blocks of consecutive rows whose bounds fit half an arena."""
         ip = req.ip_row
         cols = int(req.B.cols)
-        csum = np.cumsum(np.minimum(ip, cols) * 8 + 16)
+        # (72: a row's share of the workspace at most, of the scratch and of
+        # the row pointers)
+        csum = np.cumsum(np.minimum(ip, cols) * 8 + 72)
         target = budget // 2
         parts, r0, base = [], 0, 0
         while r0 < ip.size:

@@ -47,3 +47,21 @@ def test_narrow_rows(cols, repeats, few):
         assert nnz == int(ref.row_ptr[-1])
         cols_out = np.concatenate([C.to_host().col for _, _, C in blocks])
         assert np.array_equal(cols_out, ref.col)
+
+
+@pytest.mark.parametrize("cols", [33, 256, 1024])
+@pytest.mark.parametrize("repeats", [False, True])
+def test_narrow_rows_without_room_for_bitmaps(cols, repeats):
+    # more rows of C than the tables of a small B leave room for: both phases
+    # mark the products
+    rng = np.random.default_rng(7 * cols + repeats)
+    B = narrow_b(40, cols, repeats, rng)
+    lens = rng.choice([1, 8, 20, 33, 40, 170], size=60_000, p=[.2, .2, .2, .2, .19, .01])
+    r = np.repeat(np.arange(lens.size), lens)
+    A = gen.csr_from_coo(lens.size, B.rows, r, rng.integers(0, B.rows, size=r.size),
+                         gen.uniform_open_closed(rng, r.size), sort=False)
+    words = (cols + 31) // 32
+    assert 4 * words * lens.size > 20 * B.nnz + 8 * B.rows + 12 * (cols + 1) + 8 * 256
+    C = Plan().spgemm(DeviceCSR.from_host(A), DeviceCSR.from_host(B))
+    torch.cuda.synchronize()
+    compare(C.to_host(), oracle.spgemm(A, B))

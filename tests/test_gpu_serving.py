@@ -55,3 +55,25 @@ def test_results_same_alone_and_in_the_mix():
         compare(ha, ref)
         compare(hm, ref)
     torch.cuda.synchronize()
+
+
+def test_rows_of_few_products_split_and_counted_in_pieces():
+    # a request of many short rows: its workspace is larger than the count
+    # arena and its bound larger than a slot
+    rng = np.random.default_rng(17)
+    m, k, cols = 200_000, 1000, 20_000
+    ra = np.repeat(np.arange(m), 2)
+    A = gen.csr_from_coo(m, k, ra, rng.integers(0, k, size=ra.size), gen.uniform_open_closed(rng, ra.size))
+    rb = np.repeat(np.arange(k), 2)
+    B = gen.csr_from_coo(k, cols, rb, rng.integers(0, cols, size=rb.size), gen.uniform_open_closed(rng, rb.size))
+    srv = serving.gpu_server(slots=1, budget_bytes=12 << 20, count_ws_bytes=6 << 20, max_rows=m)
+    dA, dB = DeviceCSR.from_host(A), DeviceCSR.from_host(B)
+    req, = serving.run_served(srv, [serving.Request(A=dA, B=dB)], np.zeros(1))
+    srv.close()
+    assert req.error == 0 and len(req.result) > 1
+    assert req.ip == int(oracle.ip_count(A, B)[0].sum())
+    r0 = 0
+    for C in req.result:
+        compare(C.to_host(), oracle.spgemm(A, B, rows=np.arange(r0, r0 + C.rows)))
+        r0 += C.rows
+    assert r0 == m
