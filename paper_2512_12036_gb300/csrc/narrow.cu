@@ -150,8 +150,11 @@ __global__ void __launch_bounds__(kNarrowThreads) k_sym_narrow(CsrDev A, CsrDev 
 // What bounds it: instruction issue and the shared-memory round trip of every
 // A entry. 589,000 rows of 612 products over 256 columns: 2,013 us with
 // atomics, a bitmap marked per product and each lane emitting its own word (8
-// of 32 lanes, scattered stores), 738 us now.
-template <typename Acc>
+// of 32 lanes, scattered stores), 752 us now.
+// kBits: C's bitmaps are there (without them the row is marked here, in a
+// kernel of its own: in one kernel that code cost the other rows 752 -> 770 us
+// on 1,024 subgraphs of 256 features).
+template <typename Acc, bool kBits>
 __global__ void __launch_bounds__(kNarrowMaxWarps * 32) k_num_narrow(CsrDev A, CsrDev B,
                                                                      const int* map, Ctl* ctl,
                                                                      const int* rptC, int row_begin,
@@ -160,9 +163,9 @@ __global__ void __launch_bounds__(kNarrowMaxWarps * 32) k_num_narrow(CsrDev A, C
     extern __shared__ __align__(16) unsigned char sm_raw[];
     const int warp = threadIdx.x >> 5, lane = lane_id();
     Acc* dense = reinterpret_cast<Acc*>(sm_raw) + warp * nw * 32;
-    __shared__ unsigned s_bm[kNarrowMaxWarps][32];      // without C's bitmaps
-    unsigned* bm = s_bm[warp];
-    bm[lane] = 0u;
+    __shared__ unsigned s_bm[kBits ? 1 : kNarrowMaxWarps][32];
+    unsigned* bm = s_bm[kBits ? 0 : warp];
+    if (!kBits) bm[lane] = 0u;
     for (int c = lane; c < nw * 32; c += 32) dense[c] = Acc(0);
     __syncwarp();
     const int begin = ctl->bin_off[bin], end = ctl->bin_off[bin + 1];
@@ -180,7 +183,7 @@ __global__ void __launch_bounds__(kNarrowMaxWarps * 32) k_num_narrow(CsrDev A, C
         int rs, re;
         row_extent(A, row, rs, re, ctl);
         unsigned word = 0u;
-        if (cbits != nullptr) {
+        if (kBits) {
             if (lane < nw) word = cbits[(long long)row * nw + lane];
         } else {
             warp_expand_ahead<kWarpAhead, false>(
@@ -277,8 +280,10 @@ __global__ void __launch_bounds__(kNarrowMaxWarps * 32) k_num_narrow(CsrDev A, C
 // ---------------------------------------------------------------------------
 
 void occupancy_narrow(spgemm_plan* p) {
-    allow_max_dynamic_smem((const void*)k_num_narrow<float>, p);
-    allow_max_dynamic_smem((const void*)k_num_narrow<double>, p);
+    allow_max_dynamic_smem((const void*)k_num_narrow<float, true>, p);
+    allow_max_dynamic_smem((const void*)k_num_narrow<double, true>, p);
+    allow_max_dynamic_smem((const void*)k_num_narrow<float, false>, p);
+    allow_max_dynamic_smem((const void*)k_num_narrow<double, false>, p);
 }
 
 __global__ void k_narrow_reset(Ctl* ctl, int dup) { ctl->narrow_dup = dup; }
@@ -315,8 +320,13 @@ void launch_num_narrow(const spgemm_plan* p, bool f64, const CsrDev& A, const Cs
         SPG_LAUNCH(p, K_NUM_NARROW, s, kernel<<<grid, nwp * 32, smem, s>>>(
             A, B, w.map, w.ctl, rptC, row_begin, colC, valC, bin, nw, w.nc_bits));
     };
-    if (f64) go(k_num_narrow<double>, NB_NARROW64);
-    else go(k_num_narrow<float>, NB_NARROW32);
+    if (w.nc_bits != nullptr) {
+        if (f64) go(k_num_narrow<double, true>, NB_NARROW64);
+        else go(k_num_narrow<float, true>, NB_NARROW32);
+    } else {
+        if (f64) go(k_num_narrow<double, false>, NB_NARROW64);
+        else go(k_num_narrow<float, false>, NB_NARROW32);
+    }
 }
 
 }  // namespace spg
