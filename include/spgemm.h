@@ -306,8 +306,8 @@ int spgemm_mcl_step(const spgemm_plan* plan, const spgemm_csr* E, float theta, i
                     int32_t* col_out, float* val_out, int64_t* nnz_out, void* stream);
 
 /* --- Pruned GNN layer (Section IV-C, Eqs. 1-3): X_l = A * TopK(X_{l-1}, k) * W_l.
- * The products with the dense W_l are plain dense GEMMs and are left to the
- * caller (a BLAS); these three calls supply the sparse steps around the
+ * The products with the dense W_l are plain dense GEMMs (spgemm_dense_gemm);
+ * the calls below supply the sparse steps around the
  * SpGEMM A * TopK(X) and its backward (spgemm_backward gives the gradient on
  * TopK's pattern, i.e. M_k (.) (A^T dC) of Eq. 3). */
 
