@@ -195,7 +195,10 @@ __device__ __forceinline__ int bin_of(const GroupArgs& g, int r, bool settle) {
     const int na = g.rptA[row + 1] - g.rptA[row];
     const spgemm_opts& o = g.opts;
     if (g.phase == 0) {
-        if (ip <= 1) {
+        // settled here, but for a row of one product that the accumulation phase
+        // takes in the narrow tier: that one reads the row's bitmap, which only
+        // the allocation phase's narrow tier writes
+        if (ip < 1 || (ip == 1 && (na <= o.esc_max || g.bcols > kNarrowCols))) {
             if (settle) g.row_nnz[row] = ip < 0 ? 0 : (int)ip;
             return kSkipBin;
         }

@@ -9,7 +9,9 @@
 // are 4 bytes each. Otherwise the products are marked one by one. C's bitmap is
 // kept for the accumulation phase where the workspace has room for it (the
 // place of the dense tiers' tables, 20 bytes per entry of B); without it that
-// phase marks a row's products again.
+// phase marks a row's products again. The two phases' narrow tiers hold the
+// same rows, down to a row of one product among many A entries: the grouping
+// rules have to agree, or a row would read a bitmap that nobody wrote.
 //
 // Accumulation phase: a dense accumulator over B's columns per warp. A B row
 // without a repeated column touches every accumulator at most once, so its
