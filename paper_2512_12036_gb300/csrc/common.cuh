@@ -491,8 +491,9 @@ __device__ __forceinline__ void warp_sort(K (&v)[kN]) {
 // Block-wide ordered emit of an occupancy bitmap: the set bits of words
 // [w0, w1) of bm (bit b of word w = column c0 + 32*w + b; bits outside the
 // range to emit must be clear) become entries (column, take(32*w + b)) at
-// positions written, written+1, ... of a row
-// that starts at colC/valC + out and holds nnz_row entries. Each warp owns a
+// positions written, written+1, ... of a row that starts at colC/valC + out;
+// nothing is written at nnz_row (the row's
+// entries, or the end of a slice of it) or beyond. Each warp owns a
 // contiguous run of words; a block scan of the warps' counts places the
 // runs; inside a run, 32 words at a time, entry s of the group goes to lane
 // s mod 32, which finds its word by a search on the warp prefix of the

@@ -1302,18 +1302,20 @@ __global__ void __launch_bounds__(kHotThreads, 1) k_num_dense_hot(CsrDev A, CsrD
                 set_status(ctl, ST_INVALID);
             }
         }
-        // entries before the item's columns, and up to their end
+        // entries before the item's columns, and up to their end: the item's
+        // slice of the row, of which other blocks write the rest
         int written = 0, upto = nnz_row;
         if (q1 - q0 < kParts) {
             const int* parts = part_nnz + (size_t)row * kParts;
             bool ok = true;
-            upto = 0;
-            for (int q = 0; q < q1 && ok; ++q) {
-                if (q == q0) written = upto;
-                ok = parts[q] >= 0 && parts[q] <= nnz_row - upto;
-                if (ok) upto += parts[q];
+            int sum = 0;
+            for (int q = 0; q < kParts && ok; ++q) {
+                if (q == q0) written = sum;
+                ok = parts[q] >= 0 && parts[q] <= nnz_row - sum;
+                if (ok) sum += parts[q];
+                if (q == q1 - 1) upto = sum;
             }
-            if (!ok) {                                   // not this row's counts: write nothing
+            if (!ok || sum != nnz_row) {                 // not this row's counts: write nothing
                 set_status(ctl, ST_INTERNAL);
                 continue;
             }
@@ -1408,7 +1410,7 @@ __global__ void __launch_bounds__(kHotThreads, 1) k_num_dense_hot(CsrDev A, CsrD
                 // emit [lo, hi) in column order (bits outside it are clear)
                 written += emit_bitmap<kHotThreads>(
                     bm, (lo - pc0) >> 5, (hi - pc0 + 31) >> 5, pc0, colC, valC, out, written,
-                    nnz_row, scratch, [&](int kk) {
+                    upto, scratch, [&](int kk) {
                         const float v = st[kk];
                         st[kk] = 0.f;
                         return v;

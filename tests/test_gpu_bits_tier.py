@@ -96,3 +96,49 @@ def test_part_counts_of_another_call_are_reported():
         assert (buf[:, :1024] == -7).all() and (buf[:, 1024 + nnz:] == -7).all()
         with pytest.raises(SpgemmError):
             plan.check_status(ws, "stale part counts")
+
+
+def test_part_counts_of_the_wrong_ranges_stay_in_their_slices():
+    # counts that could be the row's but are not: a sum that is not the row's
+    # writes none of it, and a shift between two ranges leaves every entry in
+    # the slice of its own range (the blocks of a row write side by side)
+    from paper_2512_12036_gb300 import SpgemmError
+    rng = np.random.default_rng(4)
+    cols, k, parts = 300_000, 3000, 8
+    rb = np.repeat(np.arange(k), 300)
+    B = gen.csr_from_coo(k, cols, rb, rng.integers(0, cols, size=rb.size), gen.uniform_open_closed(rng, rb.size))
+    na = [1100, 2000, 2900]
+    ra = np.repeat(np.arange(len(na)), na)
+    ca = np.concatenate([rng.choice(k, size=n, replace=False) for n in na])
+    A = gen.csr_from_coo(len(na), k, ra, ca, gen.uniform_open_closed(rng, ra.size))
+    plan, dA, dB = Plan(), DeviceCSR.from_host(A), DeviceCSR.from_host(B)
+    panels = -(-cols // plan.opts["panel_cols"])
+    edge = [panels * q // parts * plan.opts["panel_cols"] for q in range(parts)] + [cols]
+    for change in ("less", "more", "down", "up"):
+        ws = plan.workspace(dA, dB)
+        ip_row, _ = plan.count(dA, dB, ws)
+        row_nnz, nnz = plan.symbolic(dA, dB, ip_row, ws)
+        rp, _ = plan.row_ptr(row_nnz, ws)
+        counts = ws[-256:].view(torch.int32)[:parts * len(na)].view(len(na), parts)
+        assert torch.equal(counts.sum(1, dtype=torch.int32), row_nnz)
+        delta = torch.zeros(parts, dtype=torch.int32, device="cuda")
+        delta[3] = -40 if change in ("less", "down") else 40
+        if change in ("down", "up"):
+            delta[4] = -delta[3]
+        counts += delta
+        buf = torch.full((2, nnz + 2048), -7, dtype=torch.int32, device="cuda")
+        col, val = buf[0, 1024:1024 + nnz], buf[1, 1024:1024 + nnz].view(torch.float32)
+        plan.numeric(dA, dB, ip_row, rp, ws, col, val)
+        torch.cuda.synchronize()
+        assert (buf[:, :1024] == -7).all() and (buf[:, 1024 + nnz:] == -7).all()
+        got, slices = col.cpu().numpy(), np.cumsum(counts.cpu().numpy(), axis=1)
+        for r, s in enumerate(rp.cpu().numpy()[:-1]):
+            if change in ("less", "more"):
+                assert (got[s:s + int(row_nnz[r])] == -7).all()
+                continue
+            for q in range(parts):
+                here = got[s + (slices[r, q - 1] if q else 0):s + slices[r, q]]
+                here = here[here != -7]
+                assert ((here >= edge[q]) & (here < edge[q + 1])).all() and here.size
+        with pytest.raises(SpgemmError):
+            plan.check_status(ws, "wrong part counts")
