@@ -142,3 +142,35 @@ def test_part_counts_of_the_wrong_ranges_stay_in_their_slices():
                 assert ((here >= edge[q]) & (here < edge[q + 1])).all() and here.size
         with pytest.raises(SpgemmError):
             plan.check_status(ws, "wrong part counts")
+
+
+@pytest.mark.parametrize("cols,panel", [(300_000, 16384), (40_000, 1024)])
+@pytest.mark.parametrize("kind", ["one_row", "every_row", "repeats"])
+def test_column_ranges_with_unsorted_b(cols, panel, kind):
+    # B rows out of order have no usable panel table: every range of a row then
+    # walks all its products and keeps those of its columns
+    rng = np.random.default_rng(cols + len(kind))
+    lens = rng.integers(100, 500, size=3000)
+    r = np.repeat(np.arange(lens.size), lens)
+    c = np.concatenate([np.sort(rng.choice(cols, size=n, replace=False)) for n in lens])
+    c[::97] = rng.integers(0, 50, size=c[::97].size)                # hot columns
+    key = np.unique(r * np.int64(cols) + c)
+    r, c = key // cols, key % cols
+    if kind == "repeats":
+        r, c = np.concatenate([r, r[::50]]), np.concatenate([c, c[::50]])
+    if kind == "one_row":
+        at = np.nonzero(r == 1700)[0]
+        c[at] = rng.permutation(c[at])
+    else:
+        p = np.lexsort((rng.random(r.size), r))
+        r, c = r[p], c[p]
+    B = gen.csr_from_coo(lens.size, cols, r, c, gen.uniform_open_closed(rng, r.size), sort=False)
+    na = [170, 900, 1100, 3000]
+    ra = np.repeat(np.arange(len(na)), na)
+    ca = np.concatenate([rng.choice(lens.size, size=n, replace=False) for n in na])
+    A = gen.csr_from_coo(len(na), lens.size, ra, ca, gen.uniform_open_closed(rng, ra.size))
+    ip, _ = oracle.ip_count(A, B)
+    assert ip.min() < 1 << 17 and ip.max() > 1 << 19
+    C = Plan(panel_cols=panel).spgemm(DeviceCSR.from_host(A), DeviceCSR.from_host(B))
+    torch.cuda.synchronize()
+    compare(C.to_host(), oracle.spgemm(A, B))
