@@ -97,12 +97,14 @@ typedef struct {
                                  one range per 128K intermediate products, at most 8 (1 to 8
                                  by the row's product count); k > 0 fixes k ranges for every
                                  row. */
-    int32_t stage_b;          /* default 0: when 1, rows of the allocation phase's block hash
-                                 tier with at most 8192 intermediate products first gather
+    int32_t stage_b;          /* default 0: when 1, the allocation phase takes the rows of its
+                                 bitmap tier (see below) in its hash tiers, and rows of the
+                                 block hash tier with at most 8192 products first gather
                                  their B row-pointer pairs and copy all their B segments into
                                  shared memory (cp.async, double-buffered over rows), then
                                  insert from there: a software form of the paper's near-memory
-                                 range-2 access (Section IV-D). Same results either way. */
+                                 range-2 access (Section IV-D). The accumulation phase is not
+                                 touched, and the results are the same either way. */
     int32_t narrow_warps;     /* default 0 (= 8): warps per block (1..16) of the narrow tiers
                                  (B with at most 1024 columns: one warp per row with a dense
                                  per-warp accumulator over B's columns) */

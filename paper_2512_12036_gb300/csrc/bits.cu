@@ -282,8 +282,8 @@ static size_t bits_num_smem(const CsrDev& B, size_t acc, bool list, int cap) {
     return (acc + (list ? 4 : 0)) * (size_t)cap + (size_t)bits_nw4(B) * (list ? 20 : 24);
 }
 
-bool bits_tier(const spgemm_plan* p, const CsrDev& B) {
-    return B.cols <= kBitsCols && B.cols > kNarrowCols && !p->opts.stage_b;
+bool bits_tier(const CsrDev& B) {
+    return B.cols <= kBitsCols && B.cols > kNarrowCols;
 }
 
 // Entries a row may have in an accumulation kernel without a column list, one

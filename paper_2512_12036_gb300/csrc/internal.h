@@ -261,7 +261,7 @@ void launch_sym_narrow(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, c
 void launch_num_narrow(const spgemm_plan* p, bool f64, const CsrDev& A, const CsrDev& B, const WsPtrs& w,
                        const int* rptC, int row_begin, int* colC, float* valC, cudaStream_t s);
 // Bitmap tiers (bits.cu).
-bool bits_tier(const spgemm_plan* p, const CsrDev& B);
+bool bits_tier(const CsrDev& B);
 int bits_cap(const spgemm_plan* p, const CsrDev& B, size_t acc);
 void launch_sym_bits(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, const WsPtrs& w,
                      int* row_nnz, int bin_lo, int bin_hi, int tier, cudaStream_t s);

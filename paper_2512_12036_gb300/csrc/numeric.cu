@@ -2001,7 +2001,7 @@ static int dense_splits(const spgemm_plan* p, int panels) {
 // entries (0: none). Rows with cached bitmaps stay in the dense tiers, which
 // read them.
 static int num_bits_cap(const spgemm_plan* p, const CsrDev& B, const WsPtrs& w) {
-    return bits_tier(p, B) && !w.rc_slot ? bits_cap(p, B, sizeof(float)) : 0;
+    return bits_tier(B) && !w.rc_slot ? bits_cap(p, B, sizeof(float)) : 0;
 }
 
 // Warp and block hash tiers: rows that outgrow the sort tier, for a B too
@@ -2113,7 +2113,7 @@ void launch_numeric_tiers(const spgemm_plan* p, const CsrDev& A, const CsrDev& B
         sort_tier(K_NUM_WARP64, k_num_sort<double, 16>, p->occ_num_sort[1][1], NB_SORT64B);
         sort_tier(K_NUM_WARP64, k_num_sort<double, 8>, p->occ_num_sort[1][0], NB_SORT64A);
     }
-    if (bits_tier(p, B)) {
+    if (bits_tier(B)) {
         // three sizes of row, so that the smaller ones leave room for more
         // blocks: up to twice warp_max_nnz, half of block_max_nnz and all
         auto bits = [&](bool f64, int lo, int hi, int tier, int cap) {

@@ -578,7 +578,8 @@ void launch_symbolic(const spgemm_plan* p, const CsrDev& A, const CsrDev& B, con
                    k_sym_sort<8><<<sms * p->occ_sym_sort[0], kSortWarps * 32, 0, s>>>(
                        A, B, w.map, w.ctl, row_nnz, SB_SORTA));
     }
-    if (bits_tier(p, B)) launch_sym_bits(p, A, B, w, row_nnz, SB_WARP, SB_BLOCK0 + SB_BLOCK_N, 0, s);
+    // (the staged tier, where asked for, is a form of the hash tiers)
+    if (bits_tier(B) && !p->opts.stage_b) launch_sym_bits(p, A, B, w, row_nnz, SB_WARP, SB_BLOCK0 + SB_BLOCK_N, 0, s);
     else if (p->opts.block_max_ip > below) launch_sym_hash(p, A, B, ip, w, row_nnz, s);
     if (B.cols <= kNarrowCols) launch_sym_narrow(p, A, B, w, row_nnz, s);
     // no more of it than B's columns need: the rest of the SM's memory is L1

@@ -68,3 +68,28 @@ def test_staged_block_tier_reports_bad_column():
     ip_row, _ = plan.count(dA, dB, ws)
     with pytest.raises(SpgemmError):
         plan.symbolic(dA, dB, ip_row, ws)
+
+
+@pytest.mark.parametrize("cols", [3000, 40000])
+def test_staging_leaves_the_accumulation_phase_alone(cols):
+    # the option stages B rows for the allocation phase only: the accumulation
+    # phase launches the same kernels with it and without
+    B = hub_matrix(3000, cols, 5, heavy_rows=set(range(0, 3000, 7)), heavy_len=300, light_deg=12)
+    A = hub_matrix(700, 3000, 6, heavy_rows={1, 50}, heavy_len=900, light_deg=60)
+    dA, dB = DeviceCSR.from_host(A), DeviceCSR.from_host(B)
+    launched = []
+    for stage_b in (0, 1):
+        plan = Plan(stage_b=stage_b)
+        ws = plan.workspace(dA, dB)
+        ip_row, _ = plan.count(dA, dB, ws)
+        row_nnz, nnz = plan.symbolic(dA, dB, ip_row, ws)
+        rp, _ = plan.row_ptr(row_nnz, ws)
+        col = torch.empty(nnz, dtype=torch.int32, device="cuda")
+        val = torch.empty(nnz, dtype=torch.float32, device="cuda")
+        plan.profile(True)
+        plan.numeric(dA, dB, ip_row, rp, ws, col, val)
+        plan.check_status(ws, "numeric")
+        launched.append({name: n for name, (_, n) in plan.profile_read().items()})
+        compare(gen.HostCSR(A.rows, cols, rp.cpu().numpy(), col.cpu().numpy(), val.cpu().numpy()),
+                oracle.spgemm(A, B))
+    assert launched[0] == launched[1]
