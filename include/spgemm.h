@@ -300,7 +300,8 @@ int spgemm_batched(const spgemm_plan* plan, const spgemm_csr* A, const spgemm_cs
  * E: rows sorted by column (as spgemm produces them). Outputs (device):
  * row_ptr_out [E.rows+1], col_out / val_out [at least min(E.nnz, E.rows*k)
  * entries] in column order. nnz_out [host, nullable]: non-NULL synchronises.
- * Workspace: spgemm_workspace_bytes for a matrix of E.rows rows.
+ * Workspace: spgemm_workspace_bytes for a matrix of E.rows rows (B with no
+ * columns); a product's workspace of as many rows does too.
  * theta <= 0, k < 0, r = 1 is a plain row normalisation (the algorithm's
  * column-stochastic start on M^T). */
 int spgemm_mcl_step(const spgemm_plan* plan, const spgemm_csr* E, float theta, int32_t k, float r,

@@ -32,8 +32,6 @@ WsLayout ws_layout(const spgemm_plan* p, long long m, long long b_rows, long lon
     off = align256(off + sizeof(int) * (size_t)kNumBins * (size_t)(L.nblk > 0 ? L.nblk : 1));
     L.scan_part = off;
     off = align256(off + sizeof(long long) * (size_t)(L.nscan + 1));
-    L.row_scratch = off;
-    off = align256(off + 3 * sizeof(int) * (size_t)(m > 0 ? m : 1));
     L.bpanel = off;
     if (L.panels > 0 && L.panels <= kMaxPanels && b_rows > 0)
         off = align256(off + sizeof(int) * (size_t)b_rows * (size_t)(L.panels + 1));
@@ -90,6 +88,10 @@ WsLayout ws_layout(const spgemm_plan* p, long long m, long long b_rows, long lon
         off = align256(off + sizeof(int) * kParts * (size_t)m);
     }
     L.total = off;
+    // the clustering step's list of rows, of which it makes do without: not
+    // asked for beside a product
+    L.row_list = off;
+    L.with_list = b_cols > 0 ? off : align256(off + sizeof(int) * (size_t)(m > 0 ? m : 1));
     return L;
 }
 
@@ -100,7 +102,6 @@ WsPtrs ws_ptrs(const WsLayout& L, void* ws, int panel_cols) {
     w.map = (int*)(b + L.map);
     w.blk_counts = (int*)(b + L.blk_counts);
     w.scan_part = (long long*)(b + L.scan_part);
-    w.row_scratch = (int*)(b + L.row_scratch);
     w.bpanel = (L.panels > 0 && L.panels <= kMaxPanels && (L.has_hot ? L.colcnt : L.total) > L.bpanel)
                    ? (int*)(b + L.bpanel) : nullptr;
     w.colcnt = L.has_hot ? (int*)(b + L.colcnt) : nullptr;
@@ -117,6 +118,7 @@ WsPtrs ws_ptrs(const WsLayout& L, void* ws, int panel_cols) {
     w.part_nnz = L.part_nnz > 0 ? (int*)(b + L.part_nnz) : nullptr;
     w.nb_bits = L.nc_bits > 0 ? (unsigned*)(b + L.nb_bits) : nullptr;
     w.nc_bits = L.nc_bits > 0 ? (unsigned*)(b + L.nc_bits) : nullptr;
+    w.row_list = nullptr;
     w.nblk = L.nblk;
     w.nscan = L.nscan;
     w.panels = L.panels;
@@ -398,7 +400,7 @@ int spgemm_workspace_bytes(const spgemm_plan* plan, const spgemm_csr* A, const s
                            size_t* bytes) {
     if (!plan || !A || !B || !bytes) return SPGEMM_ERR_INVALID;
     if (A->rows < 0 || B->rows < 0 || B->cols < 0) return SPGEMM_ERR_INVALID;
-    *bytes = ws_layout(plan, A->rows, B->rows, B->cols, B->nnz).total;
+    *bytes = ws_layout(plan, A->rows, B->rows, B->cols, B->nnz).with_list;
     return SPGEMM_OK;
 }
 
@@ -616,6 +618,7 @@ int spgemm_mcl_step(const spgemm_plan* plan, const spgemm_csr* E, float theta, i
     if (!ws || ws_bytes < L.total || ((uintptr_t)ws & 255)) return SPGEMM_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     WsPtrs w = ws_ptrs(L, ws, plan->opts.panel_cols);
+    if (ws_bytes >= L.with_list) w.row_list = (int*)((char*)ws + L.row_list);
     launch_mcl_step(plan, dev_view(E), theta, k, (double)r, order, w, row_ptr_out, col_out, val_out,
                     s);
     rc = cuda_err(cudaGetLastError());

@@ -154,7 +154,6 @@ struct WsLayout {
     size_t map = 0;          // int32 [m]
     size_t blk_counts = 0;   // int32 [kNumBins][nblk]
     size_t scan_part = 0;    // int64 [nscan + 1]
-    size_t row_scratch = 0;  // int32 [3][m]      (Markov-clustering step)
     size_t bpanel = 0;       // int32 [B.rows][P+1]  (0 bytes when P > kMaxPanels)
     size_t colcnt = 0;       // int32 [B.cols+1]  entries per column of B, then hot flags
     size_t hot_rank = 0;     // int32 [B.cols+1]  exclusive prefix of the hot flags
@@ -171,6 +170,8 @@ struct WsLayout {
     size_t nc_bits = 0;      // u32 [m][nw]       of C's (narrow tiers; 0: no room for them)
     bool has_hot = false;
     size_t total = 0;
+    size_t row_list = 0;     // int32 [m], behind the rest: rows above one warp's of the clustering
+    size_t with_list = 0;    // step, for which a workspace of rows alone has room (its bytes)
     int m = 0, nblk = 0, nscan = 0, panels = 0;
 };
 
@@ -182,7 +183,6 @@ struct WsPtrs {
     int* map;
     int* blk_counts;
     long long* scan_part;
-    int* row_scratch;
     int* bpanel;
     int* colcnt;
     int* hot_rank;
@@ -197,6 +197,7 @@ struct WsPtrs {
     int* part_nnz;           // nullptr: not counted
     unsigned* nb_bits;       // narrow tiers' bitmaps, or nullptr
     unsigned* nc_bits;
+    int* row_list;           // nullptr: no room for it
     int nblk, nscan, panels, panel_cols;
 };
 

@@ -8,9 +8,10 @@
 // inflate first). The k-th largest decision value is found by a radix
 // selection over order-preserving 32-bit keys (four 8-bit digits, a
 // 256-bin histogram each), so no sort is needed; kept entries keep their
-// column order. Selection runs once: it leaves the threshold key of every row
-// for the writing pass, which filters by it, stages the kept values in the
-// output and inflates and normalises only those. (With the selection run
+// column order. Selection runs once: it leaves a row's kept entries' count and
+// threshold key, 8 bytes in the row's places of row_ptr_out and the row map,
+// for the writing pass, which filters by the key, stages the kept values in
+// the output and inflates and normalises only those. (With the selection run
 // again before writing, and pow inlined into unrolled loops beyond the
 // instruction cache, 50,021 rows of 600 entries took 3,343 us; 511 us now.)
 // Weights and the row sum are fp64; each output is rounded once to fp32.
@@ -29,14 +30,6 @@ struct MclParams {
     int k;
     double r;
     int order;
-};
-
-// Scratch of a step: per row the k-th largest decision key and how many
-// entries equal to it are kept, and the list of rows above kMclWarpMax.
-struct MclScratch {
-    unsigned* thr;
-    int* need;
-    int* longer;
 };
 
 __device__ __forceinline__ unsigned ord_key(float x) {
@@ -68,11 +61,11 @@ __device__ __forceinline__ unsigned mcl_key(float v, const MclParams& p) {
 
 // ---------------------------------------------------------------------------
 // Selection, rows of up to kMclWarpMax entries: one warp per row. The kept
-// entries are those above the k-th largest key and the first few equal to it;
-// key and number go to the scratch, their count to counts[row]. Longer rows
-// are listed for k_mcl_select_long.
+// entries are those above a key, thr[row], and as many of the first ones equal
+// to it as counts[row] lacks then. Longer rows are left to k_mcl_select_long,
+// listed if there is a list.
 __global__ void __launch_bounds__(kMclThreads) k_mcl_select(CsrDev E, MclParams prm, int* counts,
-                                                            MclScratch ms, Ctl* ctl) {
+                                                            unsigned* thr, int* longer, Ctl* ctl) {
     constexpr int kPer = kMclWarpMax / 32;
     __shared__ int whist[kMclThreads / 32][256];
     const int lane = lane_id();
@@ -84,7 +77,7 @@ __global__ void __launch_bounds__(kMclThreads) k_mcl_select(CsrDev E, MclParams 
         row_extent(E, (int)row, s, e, ctl);
         const int n = e - s;
         if (n > kMclWarpMax) {
-            if (lane == 0) ms.longer[atomicAdd(&ctl->work[0], 1)] = (int)row;
+            if (longer && lane == 0) longer[atomicAdd(&ctl->work[0], 1)] = (int)row;
             continue;
         }
         unsigned key[kPer];
@@ -100,8 +93,7 @@ __global__ void __launch_bounds__(kMclThreads) k_mcl_select(CsrDev E, MclParams 
         }
         cnt = __reduce_add_sync(kFull, cnt);
         const bool cut = prm.k >= 0 && cnt > prm.k;
-        unsigned K = 0u;
-        int need = 0;
+        unsigned K = 0u;                                        // (0: every unpruned entry)
         if (cut) {
             // the k-th largest key by radix selection, 8 bits a pass from the
             // top, on a per-warp 256-bin histogram
@@ -126,38 +118,82 @@ __global__ void __launch_bounds__(kMclThreads) k_mcl_select(CsrDev E, MclParams 
                 __syncwarp();
                 if (above + inside == prm.k) {                  // the whole bin is kept
                     --prefix;
-                    above = prm.k;
                     break;
                 }
             }
             K = prefix;
-            need = prm.k - above;
         }
         if (lane == 0) {
             counts[row] = cut ? prm.k : cnt;
-            ms.thr[row] = K;                                    // (0: every unpruned entry)
-            ms.need[row] = need;
+            thr[row] = K;
         }
     }
 }
 
-// The same for a listed row per block: its keys in shared memory (rows of up
-// to kMclStage entries; longer ones compute them again each pass).
+// Rows of more than kMclWarpMax entries, a block each, by a counter: from the
+// list that k_mcl_select has left, or, where the workspace has no room for one,
+// from chunks of rows that are looked through. Chunks are small where there are
+// few rows, so that the blocks end together, and of a test per thread at most,
+// so that a matrix without long rows costs few steps (50,021 rows, 15% of them
+// long: the step takes 547 us with the list, 585 with chunks of 8).
+__device__ __forceinline__ int mcl_chunk(int rows, int blocks) {
+    int c = 8;
+    while (c < kMclThreads && (long long)rows > (long long)c * blocks * 8) c *= 2;
+    return c;
+}
+
+// (kList: kernels of their own, since one kernel for both took registers that
+// left room for a block less on an SM: 97 + 119 us instead of 90 + 92.)
+template <bool kList, class Row>
+__device__ __forceinline__ void mcl_long_rows(const CsrDev& E, const int* longer, int tier, Ctl* ctl,
+                                              Row&& each) {
+    __shared__ int s_next;
+    if constexpr (kList) {
+        const int n = ctl->work[0];
+        for (;;) {
+            if (threadIdx.x == 0) s_next = atomicAdd(&ctl->work[tier], 1);
+            __syncthreads();
+            if (s_next >= n) break;
+            const int row = longer[s_next];
+            int s, e;
+            row_extent(E, row, s, e, ctl);
+            each(row, s, e);                         // (with barriers)
+        }
+    } else {
+        __shared__ int s_s[kMclThreads], s_e[kMclThreads];
+        const int chunk = mcl_chunk(E.rows, gridDim.x);
+        const int t = threadIdx.x;
+        for (;;) {
+            if (t == 0) s_next = atomicAdd(&ctl->work[tier], 1);
+            __syncthreads();
+            const long long r0 = (long long)s_next * chunk;
+            if (r0 >= E.rows) break;
+            bool any = false;
+            if (t < chunk) {
+                int s = 0, e = 0;
+                if (r0 + t < E.rows) row_extent(E, (int)(r0 + t), s, e, ctl);
+                any = e - s > kMclWarpMax;
+                s_s[t] = s;
+                s_e[t] = any ? e : s;
+            }
+            if (__syncthreads_or(any))
+                for (int q = 0; q < chunk; ++q)
+                    if (s_e[q] > s_s[q]) each((int)(r0 + q), s_s[q], s_e[q]);  // (block-uniform)
+            __syncthreads();
+        }
+    }
+}
+
+// Selection of the long rows: a row's keys in shared memory (rows of up to
+// kMclStage entries; longer ones compute them again each pass).
+template <bool kList>
 __global__ void __launch_bounds__(kMclThreads) k_mcl_select_long(CsrDev E, MclParams prm, int* counts,
-                                                                 MclScratch ms, Ctl* ctl) {
+                                                                 unsigned* thr, const int* longer, Ctl* ctl) {
     __shared__ int red[33];
     __shared__ int hist[256];
-    __shared__ int s_li, s_dig, s_above, s_whole;
+    __shared__ int s_dig, s_above, s_whole;
     __shared__ unsigned skey[kMclStage];
-    const int nlong = ctl->work[0];
-    for (;;) {
-        if (threadIdx.x == 0) s_li = atomicAdd(&ctl->work[1], 1);
-        __syncthreads();
-        const int li = s_li;
-        if (li >= nlong) break;
-        const int row = ms.longer[li];
-        int s, e;
-        row_extent(E, row, s, e, ctl);
+    mcl_long_rows<kList>(E, longer, 1, ctl, [&](int row, int s, int e) {
         const int n = e - s;
         const bool staged = n <= kMclStage;
         int c0 = 0;
@@ -194,18 +230,16 @@ __global__ void __launch_bounds__(kMclThreads) k_mcl_select_long(CsrDev E, MclPa
                 above = s_above;
                 if (s_whole) {                                  // the whole bin is kept
                     --prefix;
-                    above = prm.k;
                     break;
                 }
             }
         }
         if (threadIdx.x == 0) {
             counts[row] = cut ? prm.k : cnt;
-            ms.thr[row] = prefix;
-            ms.need[row] = cut ? prm.k - above : 0;
+            thr[row] = prefix;
         }
         __syncthreads();
-    }
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -256,7 +290,7 @@ __device__ __forceinline__ double mcl_weights(const float* val, int a, int b, in
     return sum;
 }
 
-__global__ void __launch_bounds__(kMclThreads) k_mcl_write(CsrDev E, MclParams prm, MclScratch ms,
+__global__ void __launch_bounds__(kMclThreads) k_mcl_write(CsrDev E, MclParams prm, const unsigned* thr,
                                                            const int* rpt_out, int* col_out,
                                                            float* val_out, Ctl* ctl) {
     const int lane = lane_id();
@@ -266,12 +300,17 @@ __global__ void __launch_bounds__(kMclThreads) k_mcl_write(CsrDev E, MclParams p
         int s, e;
         row_extent(E, (int)row, s, e, ctl);
         if (e - s > kMclWarpMax) continue;
-        const unsigned K = ms.thr[row];
-        const int need = ms.need[row];
+        const unsigned K = thr[row];
         const int p0 = rpt_out[row], p1 = rpt_out[row + 1];
-        const bool cut = prm.k >= 0 && p1 - p0 == prm.k;
         int eq = 0;
-        const int pos = mcl_write(E, prm, K, need, cut, s, e, p0, p1, eq, col_out, val_out);
+        int pos = mcl_write(E, prm, K, 0, false, s, e, p0, p1, eq, col_out, val_out);
+        // a cut inside a run of equal values: once more, with the first of them
+        // that there is room for (the row is in L1 by now: 602 us where every
+        // row has such a cut, 597 with a second number per row in the workspace)
+        if (pos < p1 && prm.k >= 0 && p1 - p0 == prm.k) {
+            __syncwarp();                                       // (other lanes write these places now)
+            pos = mcl_write(E, prm, K, p1 - pos, true, s, e, p0, p1, eq, col_out, val_out);
+        }
         if (lane == 0 && pos != p1) set_status(ctl, ST_INTERNAL);
         __syncwarp();
         const double sum = warp_sum(mcl_weights<32>(val_out, p0, p1, lane, prm.r));
@@ -280,27 +319,18 @@ __global__ void __launch_bounds__(kMclThreads) k_mcl_write(CsrDev E, MclParams p
     }
 }
 
-// A listed row per block, a contiguous share of it per warp: every warp
-// counts the entries above and at the threshold in its share first.
-__global__ void __launch_bounds__(kMclThreads) k_mcl_write_long(CsrDev E, MclParams prm, MclScratch ms,
-                                                                const int* rpt_out, int* col_out,
-                                                                float* val_out, Ctl* ctl) {
+// A long row per block, a contiguous share of it per warp: every warp counts
+// the entries above and at the threshold in its share first.
+template <bool kList>
+__global__ void __launch_bounds__(kMclThreads) k_mcl_write_long(CsrDev E, MclParams prm, const unsigned* thr,
+                                                                const int* longer, const int* rpt_out,
+                                                                int* col_out, float* val_out, Ctl* ctl) {
     constexpr int kWarps = kMclThreads / 32;
-    __shared__ int s_li;
     __shared__ int s_gt[kWarps], s_eq[kWarps];
     __shared__ double redd[33];
     const int lane = lane_id(), warp = threadIdx.x >> 5;
-    const int nlong = ctl->work[0];
-    for (;;) {
-        if (threadIdx.x == 0) s_li = atomicAdd(&ctl->work[2], 1);
-        __syncthreads();
-        const int li = s_li;
-        if (li >= nlong) break;
-        const int row = ms.longer[li];
-        int s, e;
-        row_extent(E, row, s, e, ctl);
-        const unsigned K = ms.thr[row];
-        const int need = ms.need[row];
+    mcl_long_rows<kList>(E, longer, 2, ctl, [&](int row, int s, int e) {
+        const unsigned K = thr[row];
         const int p0 = rpt_out[row], p1 = rpt_out[row + 1];
         const bool cut = prm.k >= 0 && p1 - p0 == prm.k;
         const int per = ((e - s + kWarps - 1) / kWarps + 31) & ~31;
@@ -319,10 +349,13 @@ __global__ void __launch_bounds__(kMclThreads) k_mcl_write_long(CsrDev E, MclPar
             s_eq[warp] = at;
         }
         __syncthreads();
-        int pos = p0, eq = 0;
-        for (int w = 0; w < warp; ++w) {
-            pos += s_gt[w];
-            eq += s_eq[w];
+        int pos = p0, eq = 0, need = p1 - p0;
+        for (int w = 0; w < kWarps; ++w) {
+            need -= s_gt[w];
+            if (w < warp) {
+                pos += s_gt[w];
+                eq += s_eq[w];
+            }
         }
         if (cut) pos += eq < need ? eq : need;
         pos = mcl_write(E, prm, K, need, cut, q0, q1, pos, p1, eq, col_out, val_out);
@@ -331,8 +364,9 @@ __global__ void __launch_bounds__(kMclThreads) k_mcl_write_long(CsrDev E, MclPar
         const double sum = block_sum(mcl_weights<kMclThreads>(val_out, p0, p1, threadIdx.x, prm.r), redd);
         for (int q = p0 + (int)threadIdx.x; q < p1; q += kMclThreads)
             val_out[q] = sum > 0.0 ? (float)(mcl_weight(val_out[q], prm.r) / sum) : 0.f;
-        // (s_gt and s_li are written again after the barriers of block_sum)
-    }
+        // (s_gt is written again after the barriers of block_sum, the last of
+        // which follows every read of the row's number)
+    });
 }
 
 void launch_mcl_step(const spgemm_plan* p, const CsrDev& E, float theta, int k, double r,
@@ -343,15 +377,22 @@ void launch_mcl_step(const spgemm_plan* p, const CsrDev& E, float theta, int k, 
         return;
     }
     const MclParams prm{theta, k, r, order};
-    const MclScratch ms{(unsigned*)w.row_scratch, w.row_scratch + E.rows, w.row_scratch + 2 * (size_t)E.rows};
     const int grid = p->num_sms * 8, grid_long = p->num_sms * 6;
-    int* counts = w.map;                       // E.rows ints of the workspace
+    // the scan takes the counts in place: a thread reads its rows' counts
+    // before it writes their row pointers, and no other thread reads them then
+    int* counts = rpt_out;
+    unsigned* thr = (unsigned*)w.map;
+    int* longer = w.row_list;
     cudaMemsetAsync(w.ctl->work, 0, sizeof(w.ctl->work), s);
-    SPG_LAUNCH(p, K_MCL, s, k_mcl_select<<<grid, kMclThreads, 0, s>>>(E, prm, counts, ms, w.ctl));
-    SPG_LAUNCH(p, K_MCL, s, k_mcl_select_long<<<grid_long, kMclThreads, 0, s>>>(E, prm, counts, ms, w.ctl));
-    launch_row_ptr(p, counts, E.rows, w, rpt_out, s);
-    SPG_LAUNCH(p, K_MCL, s, k_mcl_write<<<grid, kMclThreads, 0, s>>>(E, prm, ms, rpt_out, col_out, val_out, w.ctl));
-    SPG_LAUNCH(p, K_MCL, s, k_mcl_write_long<<<grid_long, kMclThreads, 0, s>>>(E, prm, ms, rpt_out, col_out, val_out, w.ctl));
+    auto go = [&](auto select_long, auto write_long) {
+        SPG_LAUNCH(p, K_MCL, s, k_mcl_select<<<grid, kMclThreads, 0, s>>>(E, prm, counts, thr, longer, w.ctl));
+        SPG_LAUNCH(p, K_MCL, s, select_long<<<grid_long, kMclThreads, 0, s>>>(E, prm, counts, thr, longer, w.ctl));
+        launch_row_ptr(p, counts, E.rows, w, rpt_out, s);
+        SPG_LAUNCH(p, K_MCL, s, k_mcl_write<<<grid, kMclThreads, 0, s>>>(E, prm, thr, rpt_out, col_out, val_out, w.ctl));
+        SPG_LAUNCH(p, K_MCL, s, write_long<<<grid_long, kMclThreads, 0, s>>>(E, prm, thr, longer, rpt_out, col_out, val_out, w.ctl));
+    };
+    if (longer) go(k_mcl_select_long<true>, k_mcl_write_long<true>);
+    else go(k_mcl_select_long<false>, k_mcl_write_long<false>);
 }
 
 }  // namespace spg

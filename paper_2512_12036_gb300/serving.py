@@ -193,6 +193,13 @@ def request_bound(plan, A, B, ws_bytes: int, ip_total: int) -> int:
     return (int(ws_bytes) + 12 * A.rows + 4 * (A.rows + 1) + 8 * nnz_bound + 8 * 256)
 
 
+def row_bytes(plan, A, B, ws_bytes: int) -> int:
+    """Of that, what a row of A adds beside its entries of C: its share of the
+    workspace (ws_bytes, that of A*B), of the scratch and of the row pointers."""
+    per_rows = int(ws_bytes) - plan.workspace_bytes(A.view_rows(0, 0), B)
+    return 16 + -(-per_rows // max(A.rows, 1))
+
+
 class Arena:
     """Views carved from one preallocated device buffer (no allocation while
     serving); every view starts on a 256-byte boundary."""
@@ -277,9 +284,8 @@ def gpu_server(slots: int = 4, budget_bytes: int = 64 << 30, device: int = 0,
         """Blocks of consecutive rows whose bounds fit half an arena."""
         ip = req.ip_row
         cols = int(req.B.cols)
-        # (72: a row's share of the workspace at most, of the scratch and of
-        # the row pointers)
-        csum = np.cumsum(np.minimum(ip, cols) * 8 + 72)
+        nws = count_plan.workspace_bytes(req.A, req.B)
+        csum = np.cumsum(np.minimum(ip, cols) * 8 + row_bytes(count_plan, req.A, req.B, nws))
         target = budget // 2
         parts, r0, base = [], 0, 0
         while r0 < ip.size:

@@ -92,3 +92,59 @@ def test_mcl_expansions_served_match_plain_and_oracle():
     a, b = res_s.Mt.to_host(), res_p.Mt.to_host()
     assert np.array_equal(a.row_ptr, b.row_ptr) and np.array_equal(a.col, b.col)
     assert np.allclose(a.val, b.val, rtol=1e-4, atol=1e-7)
+
+
+@pytest.mark.parametrize("cols", [500, 5000, 40_000, 300_000])
+def test_product_workspace_per_row(cols):
+    # a row of A takes its place in the row map and its share of the bins'
+    # counts and the scan's; beside them, only a B that may have rows cut into
+    # column ranges takes the counts of those
+    plan = Plan()
+    B = DeviceCSR.from_host(gen.csr_from_coo(1000, cols, np.arange(1000), np.zeros(1000, int), np.ones(1000)))
+
+    def nbytes(m):
+        rp = torch.zeros(m + 1, dtype=torch.int32, device="cuda")
+        return plan.workspace_bytes(DeviceCSR(m, 1000, rp, B.col[:0], B.val[:0]), B)
+
+    m = 1 << 20
+    ranges = 32 if cols > plan.opts["panel_cols"] else 0
+    assert nbytes(2 * m) - nbytes(m) <= m * (4 + ranges) + m // 1024 * 64 * 4 + m // 4096 * 8 + 8 * 256
+
+
+def mixed_rows(rows, rng):
+    """Rows of 0 to 3,000 entries around the lengths that one warp takes, of
+    distinct values or of a few that repeat, some in no order of size."""
+    lens = rng.choice([0, 1, 5, 31, 32, 33, 127, 129], size=rows)
+    some = np.nonzero(rng.random(rows) < 40 / rows)[0]
+    lens[some] = rng.choice([1000, 1023, 1024, 1025, 1500, 3000], size=some.size)
+    lens[:2], lens[-1] = (1024, 1025), 1500
+    r = np.repeat(np.arange(rows), lens)
+    c = np.concatenate([np.sort(rng.choice(4000, size=n, replace=False)) for n in lens])
+    v = gen.uniform_open_closed(rng, r.size)
+    few = np.array([1e-5, 2e-4, 5e-4, 5e-4, 1e-3], dtype=np.float32)
+    v = np.where(np.isin(r, rng.choice(rows, size=rows // 2, replace=False)), rng.choice(few, size=r.size), v)
+    return gen.csr_from_coo(rows, 4000, r, c, v.astype(np.float32))
+
+
+@pytest.mark.parametrize("rows", [9, 700, 30_000])
+@pytest.mark.parametrize("k", [0, 1, 32, -1])
+def test_step_stays_in_the_workspace_of_its_rows(rows, k):
+    # rows of one warp and longer ones side by side, the cut inside runs of
+    # equal values, in a workspace of exactly the size that is asked for the
+    # rows alone or for a product of them with the smallest B
+    plan = Plan()
+    E = mixed_rows(rows, np.random.default_rng(rows + k))
+    dE = DeviceCSR.from_host(E)
+    none = DeviceCSR(0, 0, torch.zeros(1, dtype=torch.int32, device="cuda"), dE.col[:0], dE.val[:0])
+    small = DeviceCSR(0, 1, none.row_ptr, none.col, none.val)
+    for B in (none, small):
+        nbytes = plan.workspace_bytes(dE, B)
+        buf = plan._buffer(nbytes + 4096, dE.device).fill_(0xa5)
+        ws = buf[:nbytes]
+        plan.workspace_init(ws)
+        for order in (0, 1):
+            got = mcl_step(plan, dE, 1e-4, k, 2.0, order, ws=ws).to_host()
+            ref = oracle.mcl_step(E, 1e-4, k, 2.0, order)
+            assert np.array_equal(got.row_ptr.astype(np.int64), ref.row_ptr)
+            assert np.array_equal(got.col, ref.col) and ulp_close(got.val, ref.val)
+        assert (buf[nbytes:] == 0xa5).all()

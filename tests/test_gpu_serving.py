@@ -77,3 +77,24 @@ def test_rows_of_few_products_split_and_counted_in_pieces():
         compare(C.to_host(), oracle.spgemm(A, B, rows=np.arange(r0, r0 + C.rows)))
         r0 += C.rows
     assert r0 == m
+
+
+def test_short_rows_split_by_the_bytes_they_need():
+    # 200,000 rows of 4 products on a B without column ranges: 32 bytes of C, 16
+    # of scratch and row pointers and 4.3 of workspace a row, 10.5 MB in blocks
+    # of at most half of an 8 MiB slot
+    rng = np.random.default_rng(18)
+    m, k, cols = 200_000, 1000, 1000
+    ra = np.repeat(np.arange(m), 2)
+    A = gen.csr_from_coo(m, k, ra, rng.integers(0, k, size=ra.size), gen.uniform_open_closed(rng, ra.size))
+    rb = np.repeat(np.arange(k), 2)
+    B = gen.csr_from_coo(k, cols, rb, rng.integers(0, cols, size=rb.size), gen.uniform_open_closed(rng, rb.size))
+    srv = serving.gpu_server(slots=1, budget_bytes=8 << 20, count_ws_bytes=6 << 20, max_rows=m)
+    req, = serving.run_served(srv, [serving.Request(A=DeviceCSR.from_host(A), B=DeviceCSR.from_host(B))], np.zeros(1))
+    srv.close()
+    assert req.error == 0 and len(req.result) == -(-m * 53 // (4 << 20))
+    r0 = 0
+    for C in req.result:
+        compare(C.to_host(), oracle.spgemm(A, B, rows=np.arange(r0, r0 + C.rows)))
+        r0 += C.rows
+    assert r0 == m
