@@ -74,10 +74,21 @@ typedef struct {
 typedef struct {
     int32_t fp32_max_terms;   /* default 167: rows with more A entries accumulate in fp64 */
     int32_t esc_max;          /* default 32: IP and A-row length bound of the in-register tier */
-    int32_t warp_max_ip;      /* default 1024: allocation phase, warp-per-row hash tier */
-    int32_t block_max_ip;     /* default 16384: allocation phase, block-per-row hash tier */
-    int32_t warp_max_nnz;     /* default 512: accumulation phase, warp-per-row hash tier */
-    int32_t block_max_nnz;    /* default 8192: accumulation phase, block-per-row hash tier */
+    /* The next four bound the tiers between the in-register and the dense
+     * one. Rows of up to 512 products (allocation: at most half of
+     * warp_max_ip, accumulation: at most warp_max_nnz, where these are
+     * smaller) are sorted in a warp's registers, in the accumulation phase
+     * for a B of fewer than 2^23 columns. Larger rows take the hash tiers, or
+     * for a B of 1,025 to 2^19 columns the bitmap tiers in their place: there
+     * the four only say which launch a row is in and where the dense tiers
+     * begin (fp32 rows of the accumulation phase without cached bitmaps stay
+     * in the bitmap tier beyond that, while shared memory holds them). A B of
+     * at most 1,024 columns has the narrow tiers (below) for all of these. */
+    int32_t warp_max_ip;      /* default 1024: allocation phase, products of a row, warp per row */
+    int32_t block_max_ip;     /* default 16384: the same, block per row */
+    int32_t warp_max_nnz;     /* default 512: accumulation phase, entries of a row, warp per row
+                                 (fp32 rows of up to twice as many too) */
+    int32_t block_max_nnz;    /* default 8192: the same, block per row */
     int32_t panel_cols;       /* default 16384 (a power of two, 1024..16384): column panel of
                                  the dense heavy-row accumulator */
     int32_t row_cache_mb;     /* default 0: MiB of workspace for the allocation phase's
@@ -98,7 +109,7 @@ typedef struct {
                                  by the row's product count); k > 0 fixes k ranges for every
                                  row. */
     int32_t stage_b;          /* default 0: when 1, the allocation phase takes the rows of its
-                                 bitmap tier (see below) in its hash tiers, and rows of the
+                                 bitmap tier (see above) in its hash tiers, and rows of the
                                  block hash tier with at most 8192 products first gather
                                  their B row-pointer pairs and copy all their B segments into
                                  shared memory (cp.async, double-buffered over rows), then
@@ -111,7 +122,8 @@ typedef struct {
     int32_t narrow_max_ip;    /* default 0 (= 32768): largest IP of a row in the narrow tiers */
     int32_t hash_load_pct;    /* default 0 (= 50): target load of the hash tiers' tables in
                                  percent (25..90); a row's table is the smallest power of two
-                                 holding its keys at that load */
+                                 holding its keys at that load (the sort, bitmap and
+                                 narrow tiers have no tables) */
     int32_t reserved[3];
 } spgemm_opts;
 

@@ -492,10 +492,9 @@ __device__ __forceinline__ void warp_sort(K (&v)[kN]) {
 // [w0, w1) of bm (bit b of word w = column c0 + 32*w + b; bits outside the
 // range to emit must be clear) become entries (column, take(32*w + b)) at
 // positions written, written+1, ... of a row that starts at colC/valC + out;
-// nothing is written at nnz_row (the row's
-// entries, or the end of a slice of it) or beyond. Each warp owns a
-// contiguous run of words; a block scan of the warps' counts places the
-// runs; inside a run, 32 words at a time, entry s of the group goes to lane
+// nothing is written at nnz_row (the row's entries, or the end of a slice of
+// it) or beyond. Each warp owns a contiguous run of words; a block scan of the
+// warps' counts places the runs; inside a run, 32 words at a time, entry s of the group goes to lane
 // s mod 32, which finds its word by a search on the warp prefix of the
 // popcounts and its bit by select_bit, so the column and value stores of a
 // warp are contiguous. take(kk) returns the value and clears its slot; the
@@ -590,14 +589,13 @@ __device__ __forceinline__ int emit_bitmap_lanes(unsigned* bm, int w0, int w1, i
     return tot;
 }
 
-// The per-warp walk of expand_tile over the compacted segments. With kRun > 0,
-// kRun steps of 32 products that lie in one segment (long rows of B) are taken
-// together: one address for all of them and no test per product, which halves
-// the instructions of the allocation bitmap tier's walk (1 in 32 rows of R-MAT
-// 2^20 squared: 3,361 -> 2,595 us). (offsets
+// The per-warp walk of expand_tile over the compacted segments (offsets
 // off[0..nE], starts sbs[], multipliers sa[]). Off is int when the tile's
 // total fits 31 bits (the common case; fewer instructions per step), else
-// long long.
+// long long. With kRun > 0, kRun steps of 32 products that lie in one segment
+// (long rows of B) are taken together: one address for all of them and no test
+// per product, which halves the instructions of the allocation bitmap tier's
+// walk (1 in 32 rows of R-MAT 2^20 squared: 3,361 -> 2,595 us).
 template <typename Off, int kWarps, typename Acc, int kUnroll, bool kSeg, int kRun, class Load, class Apply>
 __device__ __forceinline__ void expand_walk(const Off* off, const int* sbsv, const Acc* sav, int nE,
                                             Off P, Load& load, Apply& apply) {

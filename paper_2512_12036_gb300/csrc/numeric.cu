@@ -4,10 +4,16 @@
 // Row tiers (bins by the row's nnz, IP and A-row length):
 //   ESC   IP <= 32: one warp, one product per lane; equal columns summed in
 //         a fixed lane order and ranked by comparison, written sorted.
-//   WARP  nnz <= 512: warp per row, (key, value) table in shared memory
-//         (Algorithm 4's AddInTable), then in-place compaction and a bitonic
-//         sort of the occupied slots.
-//   BLOCK nnz <= 8192: block per row, same scheme with a block-wide table.
+//   SORT  IP <= 512: warp per row, the products sorted in registers and runs
+//         of one column added up.
+//   NARROW, for a B of at most 1,024 columns, and bitmaps, for one of at most
+//         2^19, take the rows past these (narrow.cu, bits.cu); a wider B
+//         has the hash tiers:
+//   WARP  nnz <= 512 (fp32: 1,024): warp per row, (key, value) table in shared
+//         memory (Algorithm 4's AddInTable), then compaction to (column, slot)
+//         pairs, which are sorted in registers.
+//   BLOCK nnz <= 8192: block per row, a block-wide table, compaction and a
+//         bucket sort (a bitonic network where columns cluster).
 //   DENSE larger rows: block per row, a dense accumulator over one column
 //         panel at a time (values + occupancy bitmap in shared memory). The
 //         B entries of a panel are found through a per-B-row panel offset
@@ -110,12 +116,12 @@ __global__ void __launch_bounds__(256) k_num_esc(CsrDev A, CsrDev B, const int* 
 
 // ---------------------------------------------------------------------------
 // Bitonic sort of n2 (power of two) (key, value) pairs in shared memory,
-// ascending by key, by `nthreads` cooperating threads starting at `tid`.
-template <typename Acc, bool kBlock>
-__device__ __forceinline__ void bitonic_sort(int* keys, Acc* vals, int n2, int tid, int nthreads) {
+// ascending by key, by the block.
+template <typename Acc>
+__device__ __forceinline__ void bitonic_sort(int* keys, Acc* vals, int n2) {
     for (int k = 2; k <= n2; k <<= 1) {
         for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = tid; i < n2; i += nthreads) {
+            for (int i = threadIdx.x; i < n2; i += blockDim.x) {
                 const int ixj = i ^ j;
                 if (ixj > i) {
                     const int ki = keys[i], kj = keys[ixj];
@@ -129,8 +135,7 @@ __device__ __forceinline__ void bitonic_sort(int* keys, Acc* vals, int n2, int t
                     }
                 }
             }
-            if (kBlock) __syncthreads();
-            else __syncwarp();
+            __syncthreads();
         }
     }
 }
@@ -521,7 +526,7 @@ __global__ void __launch_bounds__(kT) k_num_block(CsrDev A, CsrDev B,
             const int n2 = (int)pow2_ceil((unsigned)(nn > 1 ? nn : 1));
             for (int t = nn + threadIdx.x; t < n2; t += blockDim.x) keys[t] = 0x7fffffff;
             __syncthreads();
-            bitonic_sort<Acc, true>(keys, vals, n2, threadIdx.x, blockDim.x);
+            bitonic_sort<Acc>(keys, vals, n2);
             so = 0;
         }
         for (int t = threadIdx.x; t < nn; t += blockDim.x) {

@@ -3,6 +3,10 @@
 // Row tiers (bins from the grouping phase):
 //   ESC   IP <= 32 and |A_i| <= 32: one warp, one product per lane; distinct
 //         columns counted with __match_any_sync, no table at all.
+//   SORT  IP <= 512: one warp per row, the columns sorted in registers.
+//   NARROW, for a B of at most 1,024 columns, and bitmaps, for one of at most
+//         2^19, take the rows past these (narrow.cu, bits.cu); a wider B
+//         has the hash tiers:
 //   WARP  IP <= 1024: one warp per row, open-addressing table of keys in
 //         shared memory (Algorithm 4's InsertIntoTable), sized 2*IP.
 //   BLOCK IP <= 16384: one block per row, shared table sized 2*IP.
